@@ -35,6 +35,7 @@ constexpr int kMaxRestart = 64;
 constexpr int kRedThreads = 256;
 constexpr int kFinThreads = 1024;   // single-block reduction / control kernels
 constexpr int kDotChunk = 16;       // basis vectors per pass of the multi-dot kernels
+constexpr int kDotLoads = 8;        // basis vectors whose values a thread has in flight at once
 
 // Krylov state of one shot
 struct ShotScalars {
@@ -45,6 +46,7 @@ struct ShotScalars {
     double H[(kMaxRestart + 1) * kMaxRestart];
     double cs[kMaxRestart], sn[kMaxRestart], g[kMaxRestart + 1], y[kMaxRestart];
     double red[3];                                // reduced sums handed between warps
+    double vscale;                                // 1 / ||w||, the scale of the next basis vector
     int jj;            // basis columns this shot uses in the current cycle
     int active;        // still iterating in the current cycle / CG solve
     int reorth;        // this Arnoldi step needs the second Gram-Schmidt pass
@@ -54,14 +56,19 @@ struct ShotScalars {
     int ir_conv, ir_zero;
 };
 
+// Recorded bodies whose executions are counted on the device: the kernels launched by a call are
+// sum_i runs[i] * (kernels of body i), the second factor known from recording.
+enum Body { kBodyStraight, kBodyIr, kBodyCycle, kBodyInner, kBodies };
+
 // loop control shared by all shots
 struct DevScalars {
     int j, iters, flag_outer, flag_inner, max_iters, m;
+    int any;           // a shot still iterates (collected by the shots' last blocks)
     int ir_flag, ir_count, ir_max;
     // statistics, reset by the host before a batch of steps
     int st_total, st_max, st_refine, st_notconv, st_nonfinite;
     double st_final_rel, st_iters_sum;
-    unsigned long long launches;      // kernel executions since the last reset
+    unsigned int runs[kBodies];       // executions of each recorded body since the last reset
 };
 
 struct Workspace {
@@ -70,10 +77,12 @@ struct Workspace {
     int64_t nvec = 0;             // values per shot (velocity DOFs)
     int64_t n = 0, ldv = 0;       // stacked length, basis leading dimension
     unsigned G = 1;               // blocks per shot of the streaming kernels (grid G x ns)
-    unsigned red_blocks = 1;      // blocks of the single-vector streaming kernels: 8 per SM
+    unsigned Gd = 1;              // blocks per shot of the multi-dot kernels
+    unsigned red_blocks = 1;      // blocks of the single-vector streaming kernels
     DevScalars* sc = nullptr;
     ShotScalars* ss = nullptr;    // [ns]
     double* partials = nullptr;   // [slot][shot][block], (kMaxRestart + 2) slots
+    unsigned* done = nullptr;     // [ns] blocks of a shot, [1] shots that have finished a reducing kernel
     double* dparams = nullptr;    // t^n, dt, step index
     double *V = nullptr, *w = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *t = nullptr;   // FP64
     float *V32 = nullptr, *w32 = nullptr, *b32 = nullptr, *x32 = nullptr, *r32 = nullptr, *p32 = nullptr, *q32 = nullptr;
@@ -84,8 +93,12 @@ struct Workspace {
     cudaGraph_t graph[2] = {};
     cudaGraphExec_t exec[2] = {};
     double graph_dt[2] = {-1.0, -1.0};
+    long body_kernels[2][kBodies] = {};   // kernels of each body, as recorded
     std::vector<void*> owned;   // device buffers of this workspace
     dim3 grid() const { return dim3(G, (unsigned)ns); }
+    dim3 dot_grid() const { return dim3(Gd, (unsigned)ns); }
+    // threads of the single-block control kernels: one per shot, at least a warp per ten shots
+    int fin_threads() const { return std::min(kFinThreads, std::max(128, (ns + 31) / 32 * 96)); }
 };
 
 static Workspace* W(stdg_ctx* c) { return reinterpret_cast<Workspace*>(c->ws); }
@@ -106,10 +119,11 @@ __device__ __forceinline__ double block_sum(double v) {
     return s;   // valid in thread 0
 }
 
-// sum of p[0..n) by one warp; valid in every lane
+// sum of p[0..n) by one warp; valid in every lane (read past L1: the values may come from other
+// blocks of the same kernel)
 __device__ __forceinline__ double warp_sum(const double* p, int n) {
     double v = 0;
-    for (int i = threadIdx.x & 31; i < n; i += 32) v += p[i];
+    for (int i = threadIdx.x & 31; i < n; i += 32) v += __ldcg(p + i);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
@@ -127,6 +141,7 @@ template <> struct Acc<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
     __device__ __forceinline__ double value() const { return s; }
+    __device__ __forceinline__ void plus_xor(const Acc& give, int o) { s += __shfl_xor_sync(0xffffffffu, give.s, o); }
 };
 template <> struct Acc<float> {
     float s = 0.f, c = 0.f;
@@ -140,7 +155,75 @@ template <> struct Acc<float> {
         c += te + pe;
     }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    // adds the pair `give` of lane ^ o (TwoSum of the leading terms): the tree over the lanes stays in
+    // float pairs, because at two FP64 lanes an SM the conversions and FP64 additions of 16 sums per
+    // thread took 5 us a block, more than the products
+    __device__ __forceinline__ void plus_xor(const Acc& give, int o) {
+        const float os = __shfl_xor_sync(0xffffffffu, give.s, o), oc = __shfl_xor_sync(0xffffffffu, give.c, o);
+        const float t = s + os;
+        const float z = t - s;
+        c += oc + ((s - (t - z)) + (os - z));
+        s = t;
+    }
 };
+
+// True in every thread of the block that arrives last of `total` (its reads then see what the
+// others wrote before arriving).  Reductions finish in that block, in a fixed order, instead of in
+// a single-block kernel of their own: a dependent launch costs 2-3 us and such a kernel took
+// 8-13 us, five of them per GMRES iteration.  The counter is back at zero afterwards.
+__device__ __forceinline__ bool last_block(unsigned* counter, unsigned total) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(counter, total - 1) == total - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Block-wide sums of the 16 accumulators that each thread holds: the lanes of a warp halve their
+// set at every exchange (16 exchanges instead of 80), then FP64 sums over the warps through shared
+// memory.  The sum of accumulator k is valid in thread k < 16.
+template <typename R>
+__device__ __forceinline__ double block_sum16(Acc<R> (&v)[kDotChunk]) {
+    __shared__ double red[32][kDotChunk];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16, n = kDotChunk / 2; o > 1; o >>= 1, n >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const Acc<R> give = up ? v[i] : v[i + n];
+            if (up) v[i] = v[i + n];
+            v[i].plus_xor(give, o);
+        }
+    }
+    v[0].plus_xor(v[0], 1);
+    const int k = (lane & 16 ? 8 : 0) + (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+    __syncthreads();
+    if ((lane & 1) == 0) red[warp][k] = v[0].value();
+    __syncthreads();
+    double s = 0;
+    if (threadIdx.x < kDotChunk)
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
+    return s;
+}
+
+// Block-wide sum of one accumulator; valid in thread 0.
+template <typename R>
+__device__ __forceinline__ double block_sum1(Acc<R> v) {
+    __shared__ double red[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v.plus_xor(v, o);
+    __syncthreads();
+    if (lane == 0) red[warp] = v.value();
+    __syncthreads();
+    double s = 0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+    return s;
+}
 
 // 16-byte vector access: VW = 4 floats or 2 doubles per load/store.  Every pointer that is
 // vectorised is 16-byte aligned (separate allocations, or basis columns at a leading
@@ -191,6 +274,12 @@ __device__ __forceinline__ void put_partial(double* part, int k, double v) {
     if (threadIdx.x == 0) part[((int64_t)k * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
 }
 
+template <typename R>
+__device__ __forceinline__ void put_acc(double* part, int k, const Acc<R>& v) {
+    const double s = block_sum1(v);
+    if (threadIdx.x == 0) part[((int64_t)k * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
+}
+
 __device__ __forceinline__ void set_cond(cudaGraphConditionalHandle h, int use, int v) {
     if (use) cudaGraphSetConditional(h, v ? 1u : 0u);
 }
@@ -203,7 +292,7 @@ __global__ void dot_partial_kernel(int64_t nvec, const A* __restrict__ a, const 
     const int64_t lo = (int64_t)blockIdx.y * nvec;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvec; i += (int64_t)gridDim.x * blockDim.x)
         acc.add(a[lo + i], b[lo + i]);
-    put_partial(part, k, acc.value());
+    put_acc(part, k, acc);
 }
 
 // x_s = 0 for the shots whose right-hand side is zero (level 0: Krylov, 1: refinement)
@@ -272,18 +361,26 @@ __global__ void copy_kernel(int64_t n, const R* __restrict__ a, R* __restrict__ 
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) b[i] = a[i];
 }
 
-// alpha_s = (r.z)_s / (p.q)_s for the shots still iterating, 0 for the frozen ones
-__global__ void __launch_bounds__(kFinThreads) cg_alpha_kernel(ShotScalars* ss, const double* part, int ns, int G) {
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int s = warp; s < ns; s += nw) {
-        const double pq = warp_sum(slot(part, 0, s, ns, G), G);
-        if ((threadIdx.x & 31) == 0) ss[s].alpha = ss[s].active && pq != 0.0 ? ss[s].pq / pq : 0.0;
-    }
+// p.q of each shot; the shot's last block forms alpha_s = (r.z)_s / (p.q)_s (0 for a frozen shot)
+template <typename R>
+__global__ void cg_dot_alpha_kernel(int64_t nvec, const R* __restrict__ p, const R* __restrict__ q, double* part,
+                                    ShotScalars* ss, unsigned* done) {
+    const int s = blockIdx.y, G = gridDim.x;
+    if (!ss[s].active) return;
+    Acc<R> acc;
+    const int64_t lo = (int64_t)s * nvec;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvec; i += (int64_t)G * blockDim.x)
+        acc.add(p[lo + i], q[lo + i]);
+    put_acc(part, 0, acc);
+    if (!last_block(done + s, G) || threadIdx.x >= 32) return;
+    const double pq = warp_sum(slot(part, 0, s, gridDim.y, G), G);
+    if (threadIdx.x == 0) ss[s].alpha = pq != 0.0 ? ss[s].pq / pq : 0.0;
 }
 
 template <typename R>
 __global__ void cg_update_kernel(int64_t nvec, const ShotScalars* __restrict__ ss, R* __restrict__ x, R* __restrict__ r,
                                  const R* __restrict__ p, const R* __restrict__ q, double* __restrict__ part) {
+    if (!ss[blockIdx.y].active) return;
     const double a = ss[blockIdx.y].alpha;
     const int64_t lo = (int64_t)blockIdx.y * nvec;
     double rr = 0;
@@ -296,40 +393,45 @@ __global__ void cg_update_kernel(int64_t nvec, const ShotScalars* __restrict__ s
     put_partial(part, 0, rr);
 }
 
-// slots: 0 rr, 2 rz (r.z after the preconditioner)
-__global__ void __launch_bounds__(kFinThreads) cg_beta_kernel(DevScalars* sc, ShotScalars* ss, const double* part, int ns,
-                                                              int G, cudaGraphConditionalHandle h, int use_h) {
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int q = warp; q < 2 * ns; q += nw) {
-        const int k = q % 2 == 0 ? 0 : 2;
-        const double v = warp_sum(slot(part, k, q / 2, ns, G), G);
-        if ((threadIdx.x & 31) == 0) ss[q / 2].red[k] = v;
+// r.z of each shot (slot 2; slot 0 holds the parts of r.r); the shot's last block forms beta_s and
+// the convergence test, and the last shot to get there advances the loop
+template <typename R>
+__global__ void cg_dot_beta_kernel(int64_t nvec, const R* __restrict__ r, const R* __restrict__ z, double* part,
+                                   DevScalars* sc, ShotScalars* ss, unsigned* done, cudaGraphConditionalHandle h, int use_h) {
+    const int s = blockIdx.y, ns = gridDim.y, G = gridDim.x;
+    ShotScalars& t = ss[s];
+    if (t.active) {
+        Acc<R> acc;
+        const int64_t lo = (int64_t)s * nvec;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvec; i += (int64_t)G * blockDim.x)
+            acc.add(r[lo + i], z[lo + i]);
+        put_acc(part, 2, acc);
     }
-    __syncthreads();
-    int any = 0;
-    for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-        ShotScalars& t = ss[s];
-        if (t.active) {
-            const double rz = t.red[2];
+    if (!last_block(done + s, G) || threadIdx.x >= 32) return;
+    if (t.active) {
+        const double rr = warp_sum(slot(part, 0, s, ns, G), G);
+        const double rz = warp_sum(slot(part, 2, s, ns, G), G);
+        if (threadIdx.x == 0) {
             t.beta = t.pq != 0.0 ? rz / t.pq : 0.0;
             t.pq = rz;
-            t.rr = t.red[0];
-            t.converged = sqrt(t.rr) <= t.tol_abs;
-            t.active = !t.converged && isfinite(t.rr);
+            t.rr = rr;
+            t.converged = sqrt(rr) <= t.tol_abs;
+            t.active = !t.converged && isfinite(rr);
         }
-        if (!t.active) t.beta = 0.0;
-        any |= t.active;
     }
-    any = __syncthreads_or(any);
-    if (threadIdx.x == 0) {
-        sc->iters += 1;
-        sc->flag_inner = any && sc->iters < sc->max_iters;
-        set_cond(h, use_h, sc->flag_inner);
-    }
+    if (threadIdx.x != 0) return;
+    if (t.active) atomicOr(&sc->any, 1);
+    __threadfence();
+    if (atomicInc(done + ns, ns - 1) != (unsigned)ns - 1) return;
+    sc->iters += 1;
+    sc->runs[kBodyInner] += 1;
+    sc->flag_inner = atomicExch(&sc->any, 0) && sc->iters < sc->max_iters;
+    set_cond(h, use_h, sc->flag_inner);
 }
 
 template <typename R>
 __global__ void cg_p_kernel(int64_t nvec, const ShotScalars* __restrict__ ss, const R* __restrict__ z, R* __restrict__ p) {
+    if (!ss[blockIdx.y].active) return;
     const double b = ss[blockIdx.y].beta;
     const int64_t lo = (int64_t)blockIdx.y * nvec;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvec; i += (int64_t)gridDim.x * blockDim.x)
@@ -339,9 +441,12 @@ __global__ void cg_p_kernel(int64_t nvec, const ShotScalars* __restrict__ ss, co
 // ---------------------------------------------------------------------------------
 // GMRES kernels (one Arnoldi process and one Hessenberg matrix per shot)
 // ---------------------------------------------------------------------------------
+// r = b - A x into v0; with start != 0 the last block of each shot also opens a restart cycle:
+// beta_s = ||r_s|| (the true residual), convergence test, g = beta_s e_1
 template <typename R>
 __global__ void gm_res_kernel(int64_t nvec, const R* __restrict__ b, const R* __restrict__ Ax, R* __restrict__ v0,
-                             double* __restrict__ part) {
+                             double* __restrict__ part, int start, DevScalars* sc, ShotScalars* ss, unsigned* done,
+                             cudaGraphConditionalHandle h, int use_h) {
     constexpr int VW = VL<R>::W;
     Acc<R> rr;
     seg_loop<R>(nvec,
@@ -354,7 +459,28 @@ __global__ void gm_res_kernel(int64_t nvec, const R* __restrict__ b, const R* __
             VL<R>::st(v0 + i, bb);
         },
         [&](int64_t i) { const R ri = b[i] - Ax[i]; v0[i] = ri; rr.add(ri, ri); });
-    put_partial(part, 0, rr.value());
+    put_acc(part, 0, rr);
+    if (!start) return;
+    const int s = blockIdx.y, ns = gridDim.y, G = gridDim.x;
+    if (!last_block(done + s, G)) return;
+    ShotScalars& t = ss[s];
+    for (int k = threadIdx.x; k <= sc->m; k += blockDim.x) t.g[k] = 0.0;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const double beta = sqrt(warp_sum(slot(part, 0, s, ns, G), G));
+    if (threadIdx.x != 0) return;
+    t.gbeta = beta;
+    t.resid = beta;
+    t.jj = 0;
+    if (!t.converged) t.converged = beta <= t.tol_abs;
+    t.active = !t.converged && isfinite(beta) && isfinite(t.tol_abs);   // a NaN/Inf residual stops the shot
+    t.g[0] = beta;
+    if (t.active) atomicOr(&sc->any, 1);
+    __threadfence();
+    if (atomicInc(done + ns, ns - 1) != (unsigned)ns - 1) return;
+    sc->j = 0;
+    sc->flag_inner = atomicExch(&sc->any, 0) && sc->iters < sc->max_iters;
+    set_cond(h, use_h, sc->flag_inner);
 }
 
 // set up one GMRES solve: ||b_s|| (from slot 0, or given), tolerances, counters
@@ -392,38 +518,6 @@ __global__ void __launch_bounds__(kFinThreads) gm_init_kernel(DevScalars* sc, Sh
     }
 }
 
-// restart: beta_s = ||r_s|| (the true residual), convergence test, g = beta_s e_1
-__global__ void __launch_bounds__(kFinThreads) gm_cycle_start_kernel(DevScalars* sc, ShotScalars* ss, const double* part,
-                                                                     int ns, int G, cudaGraphConditionalHandle h,
-                                                                     int use_h) {
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int s = warp; s < ns; s += nw) {
-        const double v = warp_sum(slot(part, 0, s, ns, G), G);
-        if ((threadIdx.x & 31) == 0) ss[s].red[0] = v;
-    }
-    __syncthreads();
-    const int m = sc->m;
-    int any = 0;
-    for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-        ShotScalars& t = ss[s];
-        const double beta = sqrt(t.red[0]);
-        t.gbeta = beta;
-        t.resid = beta;
-        t.jj = 0;
-        if (!t.converged) t.converged = beta <= t.tol_abs;
-        t.active = !t.converged && isfinite(beta) && isfinite(t.tol_abs);   // a NaN/Inf residual stops the shot
-        for (int k = 0; k <= m; ++k) t.g[k] = 0.0;
-        t.g[0] = beta;
-        any |= t.active;
-    }
-    any = __syncthreads_or(any);
-    if (threadIdx.x == 0) {
-        sc->j = 0;
-        sc->flag_inner = any && sc->iters < sc->max_iters;
-        set_cond(h, use_h, sc->flag_inner);
-    }
-}
-
 template <typename R>
 __global__ void gm_scale0_kernel(int64_t nvec, const DevScalars* __restrict__ sc, const ShotScalars* __restrict__ ss,
                                  R* __restrict__ v0) {
@@ -442,83 +536,142 @@ __global__ void gm_scale0_kernel(int64_t nvec, const DevScalars* __restrict__ sc
         [&](int64_t i) { v0[i] *= s; });
 }
 
-// slot k, shot s: sum_i V_k[i] w[i] over the shot's segment, k = 0..j (basis columns at stride ldv)
+// Accumulates V_k . w over the values at i for the kn <= kDotChunk columns from k0.  The columns
+// are loaded kDotLoads at a time before the first is used: with one 16-byte load per column in
+// flight the kernel waited on memory (long scoreboard) at 0.4-0.5 of the DRAM rate.
+template <typename R, int VW>
+__device__ __forceinline__ void dot_columns(const R* __restrict__ V, int64_t ldv, int64_t i, int kn, const R (&wv)[VW],
+                                            Acc<R> (&acc)[kDotChunk]) {
+#pragma unroll
+    for (int g = 0; g < kDotChunk; g += kDotLoads) {
+        if (g >= kn) break;
+        R vv[kDotLoads][VW];
+#pragma unroll
+        for (int kk = 0; kk < kDotLoads; ++kk)
+            if (g + kk < kn) VL<R>::ld(V + (int64_t)(g + kk) * ldv + i, vv[kk]);
+#pragma unroll
+        for (int kk = 0; kk < kDotLoads; ++kk)
+            if (g + kk < kn) {
+#pragma unroll
+                for (int u = 0; u < VW; ++u) acc[g + kk].add(vv[kk][u], wv[u]);
+            }
+    }
+}
+
+// the block's sums of acc[0..kn) into slots k0.. of its shot
 template <typename R>
-__global__ void __launch_bounds__(256, 4) gm_mdot_kernel(int64_t nvec, int64_t ldv, const DevScalars* __restrict__ sc,
-                                                      const R* __restrict__ V, const R* __restrict__ w,
-                                                      double* __restrict__ part) {
+__device__ __forceinline__ void put_chunk(double* part, int k0, int kn, Acc<R> (&acc)[kDotChunk]) {
+    const double s = block_sum16(acc);
+    if ((int)threadIdx.x < kn) part[((int64_t)(k0 + threadIdx.x) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
+}
+
+// v[i] - sum_k h_k V_k[i], four columns loaded before the first is used
+template <typename R, int VW>
+__device__ __forceinline__ void subtract_columns(const R* __restrict__ V, int64_t ldv, int64_t i, int n, const R* h,
+                                                 R (&wv)[VW]) {
+    int k = 0;
+    for (; k + 4 <= n; k += 4) {
+        R vv[4][VW];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) VL<R>::ld(V + (int64_t)(k + q) * ldv + i, vv[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < VW; ++u) wv[u] = fma(-h[k + q], vv[q][u], wv[u]);
+    }
+    for (; k < n; ++k) {
+        R vv[VW];
+        VL<R>::ld(V + (int64_t)k * ldv + i, vv);
+#pragma unroll
+        for (int u = 0; u < VW; ++u) wv[u] = fma(-h[k], vv[u], wv[u]);
+    }
+}
+
+// First classical Gram-Schmidt pass: V_k . w (k = 0..j) and ||w||^2 of every shot still iterating;
+// the shot's last block sums the blocks' parts, starts the Hessenberg column and decides whether
+// the second pass is needed: one pass leaves w orthogonal to the basis to about
+// eps ||w|| / ||w - V h||, so the pass is repeated when that ratio would exceed 10, i.e. when
+// ||w - V h||^2 = ||w||^2 - |h|^2 < 1e-2 ||w||^2 (V orthonormal; the dots are FP64-accurate).
+// The grid is sized by the vector: one 16-byte item a thread, at most two blocks an SM (128
+// registers, eight columns in flight a thread).  Measured with 13 FP64 columns of 291,600 values:
+// 24 us, where a fixed grid of 1,216 blocks with one block-wide reduction per column and a
+// single-block final kernel took 78 + 13 us; with ten FP32 columns of 16,056,320 values 127 us
+// (5.6 TB/s) against 210 + 13 us.  Short vectors stay at the chain of its dependent accesses, 8 us.
+template <typename R>
+__global__ void __launch_bounds__(256, 2) gm_mdot_kernel(int64_t nvec, int64_t ldv, const DevScalars* __restrict__ sc,
+                                                      ShotScalars* ss, const R* __restrict__ V, const R* __restrict__ w,
+                                                      double* part, unsigned* done) {
     constexpr int VW = VL<R>::W;
-    const int J = sc->j;
+    const int J = sc->j, s = blockIdx.y, ns = gridDim.y, G = gridDim.x;
+    if (!ss[s].active) return;
     for (int k0 = 0; k0 <= J; k0 += kDotChunk) {
         Acc<R> acc[kDotChunk];
         Acc<R> ww;                                // ||w||^2, first chunk only
         const int kn = min(kDotChunk, J + 1 - k0);
+        const R* Vk = V + (int64_t)k0 * ldv;
         seg_loop<R>(nvec,
             [&](int64_t i) {
                 R wv[VW];
                 VL<R>::ld(w + i, wv);
+                dot_columns<R, VW>(Vk, ldv, i, kn, wv, acc);
                 if (k0 == 0) {
 #pragma unroll
                     for (int u = 0; u < VW; ++u) ww.add(wv[u], wv[u]);
                 }
-#pragma unroll
-                for (int kk = 0; kk < kDotChunk; ++kk)
-                    if (kk < kn) {
-                        R vv[VW];
-                        VL<R>::ld(V + (int64_t)(k0 + kk) * ldv + i, vv);
-#pragma unroll
-                        for (int u = 0; u < VW; ++u) acc[kk].add(vv[u], wv[u]);
-                    }
             },
             [&](int64_t i) {
                 if (k0 == 0) ww.add(w[i], w[i]);
 #pragma unroll
                 for (int kk = 0; kk < kDotChunk; ++kk)
-                    if (kk < kn) acc[kk].add(V[(int64_t)(k0 + kk) * ldv + i], w[i]);
+                    if (kk < kn) acc[kk].add(Vk[(int64_t)kk * ldv + i], w[i]);
             });
-#pragma unroll
-        for (int kk = 0; kk < kDotChunk; ++kk)   // constant bound keeps acc[] in registers
-            if (kk < kn) put_partial(part, k0 + kk, acc[kk].value());   // kn is uniform over the block
-        if (k0 == 0) put_partial(part, J + 1, ww.value());
+        put_chunk<R>(part, k0, kn, acc);
+        if (k0 == 0) put_acc(part, J + 1, ww);
     }
+    if (!last_block(done + s, G)) return;
+    ShotScalars& t = ss[s];
+    __shared__ double h[kMaxRestart + 2];
+    for (int k = threadIdx.x >> 5; k <= J + 1; k += blockDim.x >> 5) {
+        const double v = warp_sum(slot(part, k, s, ns, G), G);
+        if ((threadIdx.x & 31) == 0) {
+            h[k] = v;
+            if (k <= J) t.hpass[k] = t.hcol[k] = v;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double h2 = 0.0;
+    for (int k = threadIdx.x; k <= J; k += 32) h2 += h[k] * h[k];
+    for (int o = 16; o > 0; o >>= 1) h2 += __shfl_xor_sync(0xffffffffu, h2, o);
+    if (threadIdx.x == 0) t.reorth = h[J + 1] - h2 < 1e-2 * h[J + 1];
 }
 
-// Second Gram-Schmidt pass fused with the first subtraction:
-// w_s <- w_s - sum_k h1_s[k] V_k, then partials of V_k . w_s for the re-orthogonalisation.
+// Second Gram-Schmidt pass fused with the first subtraction, only for the shots that need it:
+// w_s <- w_s - sum_k h1_s[k] V_k, then V_k . w_s for the re-orthogonalisation; the shot's last
+// block adds the second pass to the Hessenberg column.
 template <typename R>
-__global__ void __launch_bounds__(256, 3) gm_orth_fused_kernel(int64_t nvec, int64_t ldv, const DevScalars* __restrict__ sc,
-                                                            const ShotScalars* __restrict__ ss, const R* __restrict__ V,
-                                                            R* __restrict__ w, double* __restrict__ part) {
+__global__ void __launch_bounds__(256, 2) gm_orth_fused_kernel(int64_t nvec, int64_t ldv, const DevScalars* __restrict__ sc,
+                                                            ShotScalars* ss, const R* __restrict__ V,
+                                                            R* __restrict__ w, double* part, unsigned* done) {
     constexpr int VW = VL<R>::W;
-    const int J = sc->j;
-    if (!ss[blockIdx.y].reorth) return;           // this shot's first pass was enough
+    const int J = sc->j, s = blockIdx.y, ns = gridDim.y, G = gridDim.x;
+    if (!ss[s].active || !ss[s].reorth) return;   // this shot's first pass was enough
     __shared__ R h[kMaxRestart + 2];
-    for (int k = threadIdx.x; k <= J; k += blockDim.x) h[k] = (R)ss[blockIdx.y].hpass[k];
+    for (int k = threadIdx.x; k <= J; k += blockDim.x) h[k] = (R)ss[s].hpass[k];
     __syncthreads();
     for (int k0 = 0; k0 <= J; k0 += kDotChunk) {
         Acc<R> acc[kDotChunk];
         const int kn = min(kDotChunk, J + 1 - k0);
+        const R* Vk = V + (int64_t)k0 * ldv;
         seg_loop<R>(nvec,
             [&](int64_t i) {
                 R wv[VW];
                 VL<R>::ld(w + i, wv);
                 if (k0 == 0) {   // first chunk: form and store the projected w (in the vector precision)
-                    for (int k = 0; k <= J; ++k) {
-                        R vv[VW];
-                        VL<R>::ld(V + (int64_t)k * ldv + i, vv);
-#pragma unroll
-                        for (int u = 0; u < VW; ++u) wv[u] = fma(-h[k], vv[u], wv[u]);
-                    }
+                    subtract_columns<R, VW>(V, ldv, i, J + 1, h, wv);
                     VL<R>::st(w + i, wv);
                 }
-#pragma unroll
-                for (int kk = 0; kk < kDotChunk; ++kk)
-                    if (kk < kn) {
-                        R vv[VW];
-                        VL<R>::ld(V + (int64_t)(k0 + kk) * ldv + i, vv);
-#pragma unroll
-                        for (int u = 0; u < VW; ++u) acc[kk].add(vv[u], wv[u]);
-                    }
+                dot_columns<R, VW>(Vk, ldv, i, kn, wv, acc);
             },
             [&](int64_t i) {
                 R wi = w[i];
@@ -528,99 +681,129 @@ __global__ void __launch_bounds__(256, 3) gm_orth_fused_kernel(int64_t nvec, int
                 }
 #pragma unroll
                 for (int kk = 0; kk < kDotChunk; ++kk)
-                    if (kk < kn) acc[kk].add(V[(int64_t)(k0 + kk) * ldv + i], wi);
+                    if (kk < kn) acc[kk].add(Vk[(int64_t)kk * ldv + i], wi);
             });
-#pragma unroll
-        for (int kk = 0; kk < kDotChunk; ++kk)
-            if (kk < kn) put_partial(part, k0 + kk, acc[kk].value());
+        put_chunk<R>(part, k0, kn, acc);
     }
-}
-
-// hpass_s[k] = reduced slot k (k = 0..j); pass 0 starts the Hessenberg column, pass 1 adds
-// Pass 0 also decides, per shot, whether the second pass is needed: one classical
-// Gram-Schmidt pass leaves w orthogonal to the basis to about eps ||w|| / ||w - V h||, so the
-// pass is repeated when that ratio would exceed 10, i.e. when
-// ||w - V h||^2 = ||w||^2 - |h|^2 < 1e-2 ||w||^2 (V orthonormal; the dots are FP64-accurate).
-__global__ void __launch_bounds__(kFinThreads) gm_mdot_final_kernel(const DevScalars* sc, ShotScalars* ss,
-                                                                    const double* part, int ns, int G, int pass) {
-    const int J = sc->j;
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nk = pass == 0 ? J + 2 : J + 1;    // pass 0: slot J+1 holds ||w||^2
-    for (int q = warp; q < nk * ns; q += nw) {
-        const int k = q / ns, s = q % ns;
-        if (pass == 1 && !ss[s].reorth) continue;
+    if (!last_block(done + s, G)) return;
+    ShotScalars& t = ss[s];
+    for (int k = threadIdx.x >> 5; k <= J; k += blockDim.x >> 5) {
         const double v = warp_sum(slot(part, k, s, ns, G), G);
         if ((threadIdx.x & 31) == 0) {
-            if (k <= J) {
-                ss[s].hpass[k] = v;
-                ss[s].hcol[k] = pass == 0 ? v : ss[s].hcol[k] + v;
-            } else {
-                ss[s].red[0] = v;
-            }
+            t.hpass[k] = v;
+            t.hcol[k] += v;
         }
     }
-    if (pass != 0) return;
-    __syncthreads();
-    for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-        ShotScalars& t = ss[s];
-        double h2 = 0.0;
-        for (int k = 0; k <= J; ++k) h2 += t.hcol[k] * t.hcol[k];
-        t.reorth = t.red[0] - h2 < 1e-2 * t.red[0];
-    }
 }
 
-// w_s -= sum_k hpass_s[k] V_k; partial ||w_s||^2 into slot 0
+// w_s -= sum_k hpass_s[k] V_k and ||w_s||.  The shot's last block closes the Arnoldi step: Givens
+// rotations of the new Hessenberg column, residual estimate; the shot stops at its residual
+// estimate or on breakdown and keeps the columns it has (jj).  The last shot to get there advances
+// the loop.  For short vectors the kernel is a chain of dependent memory accesses (about 0.6 us
+// each), so everything that the closing needs is loaded beside the coefficients, before the vector:
+// 9 us for 2,352 values, against 18 + 9 + 10 us for the subtraction and its two single-block kernels.
 template <typename R>
-__global__ void __launch_bounds__(256) gm_maxpy_kernel(int64_t nvec, int64_t ldv, const DevScalars* __restrict__ sc,
-                                                       const ShotScalars* __restrict__ ss, const R* __restrict__ V,
-                                                       R* __restrict__ w, double* __restrict__ part) {
+__global__ void __launch_bounds__(256) gm_maxpy_kernel(int64_t nvec, int64_t ldv, DevScalars* sc, ShotScalars* ss,
+                                                       const R* __restrict__ V, R* __restrict__ w, double* part,
+                                                       unsigned* done, cudaGraphConditionalHandle handle, int use_h) {
     constexpr int VW = VL<R>::W;
-    const int J = sc->j;
+    const int J = sc->j, s = blockIdx.y, ns = gridDim.y, G = gridDim.x;
+    const int iters = sc->iters, max_iters = sc->max_iters, m = sc->m;
+    const unsigned runs = sc->runs[kBodyInner];
     __shared__ R h[kMaxRestart + 2];
-    for (int k = threadIdx.x; k <= J; k += blockDim.x) h[k] = (R)ss[blockIdx.y].hpass[k];
-    __syncthreads();
-    Acc<R> nn;
-    seg_loop<R>(nvec,
-        [&](int64_t i) {
-            R wv[VW];
-            VL<R>::ld(w + i, wv);
-            for (int k = 0; k <= J; ++k) {
-                R vv[VW];
-                VL<R>::ld(V + (int64_t)k * ldv + i, vv);
+    __shared__ double hc[kMaxRestart + 2], cs[kMaxRestart], sn[kMaxRestart];
+    ShotScalars& t = ss[s];
+    int active = t.active;
+    const double g = t.g[J], tol = t.tol_abs;
+    if (active) {
+        for (int k = threadIdx.x; k <= J; k += blockDim.x) {
+            h[k] = (R)t.hpass[k];
+            hc[k] = t.hcol[k];
+            cs[k] = t.cs[k];
+            sn[k] = t.sn[k];
+        }
+        __syncthreads();
+        Acc<R> nn;
+        seg_loop<R>(nvec,
+            [&](int64_t i) {
+                R wv[VW];
+                VL<R>::ld(w + i, wv);
+                subtract_columns<R, VW>(V, ldv, i, J + 1, h, wv);
+                VL<R>::st(w + i, wv);
 #pragma unroll
-                for (int u = 0; u < VW; ++u) wv[u] = fma(-h[k], vv[u], wv[u]);
-            }
-            VL<R>::st(w + i, wv);
-#pragma unroll
-            for (int u = 0; u < VW; ++u) nn.add(wv[u], wv[u]);
-        },
-        [&](int64_t i) {
-            R wi = w[i];
-            for (int k = 0; k <= J; ++k) wi = fma(-h[k], V[(int64_t)k * ldv + i], wi);
-            w[i] = wi;
-            nn.add(wi, wi);
-        });
-    put_partial(part, 0, nn.value());
-}
-
-__global__ void __launch_bounds__(kFinThreads) gm_norm_final_kernel(const DevScalars* sc, ShotScalars* ss, const double* part,
-                                                                    int ns, int G) {
-    const int J = sc->j;
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int s = warp; s < ns; s += nw) {
-        const double v = warp_sum(slot(part, 0, s, ns, G), G);
-        if ((threadIdx.x & 31) == 0) ss[s].hcol[J + 1] = sqrt(v);
+                for (int u = 0; u < VW; ++u) nn.add(wv[u], wv[u]);
+            },
+            [&](int64_t i) {
+                R wi = w[i];
+                for (int k = 0; k <= J; ++k) wi = fma(-h[k], V[(int64_t)k * ldv + i], wi);
+                w[i] = wi;
+                nn.add(wi, wi);
+            });
+        put_acc(part, 0, nn);
     }
+    if (!last_block(done + s, G)) return;
+    if (active) {
+        double v = 0;
+        const double* p = slot(part, 0, s, ns, G);
+        for (int i = threadIdx.x; i < G; i += blockDim.x) v += __ldcg(p + i);
+        v = block_sum(v);   // ||w||^2 in thread 0
+        if (threadIdx.x < 32) {
+            v = __shfl_sync(0xffffffffu, v, 0);
+            double hi = hc[0];
+            for (int i = 0; i < J; ++i) {   // every lane alike
+                const double hn = hc[i + 1];
+                const double u = cs[i] * hi + sn[i] * hn;
+                hi = -sn[i] * hi + cs[i] * hn;
+                __syncwarp();
+                if (threadIdx.x == 0) hc[i] = u;
+            }
+            // one square root and one division for the warp: lane 0 the rotated diagonal, lane 1 ||w||
+            const double root = sqrt(threadIdx.x == 0 ? fma(hi, hi, v) : v);
+            const double den = __shfl_sync(0xffffffffu, root, 0), b = __shfl_sync(0xffffffffu, root, 1);
+            const double bot = threadIdx.x == 2 ? b : den;
+            const double quo = (threadIdx.x == 0 ? hi : threadIdx.x == 1 ? b : 1.0) / (bot > 0.0 ? bot : 1.0);
+            const double q0 = __shfl_sync(0xffffffffu, quo, 0), q1 = __shfl_sync(0xffffffffu, quo, 1);
+            const double q2 = __shfl_sync(0xffffffffu, quo, 2);
+            const double c = den > 0.0 ? q0 : 1.0, q = den > 0.0 ? q1 : 0.0, resid = fabs(q * g);
+            if (resid <= tol || den == 0.0 || !isfinite(resid)) active = 0;
+            if (threadIdx.x == 0) {
+                hc[J] = den;
+                t.cs[J] = c;
+                t.sn[J] = q;
+                t.vscale = b > 0.0 ? q2 : 0.0;
+                t.g[J + 1] = -q * g;
+                t.g[J] = c * g;
+                t.resid = resid;
+                t.jj = J + 1;
+                t.active = active;
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i <= J; i += blockDim.x) t.H[i * kMaxRestart + J] = hc[i];
+    }
+    if (threadIdx.x != 0) return;
+    if (ns > 1) {
+        if (active) atomicOr(&sc->any, 1);
+        __threadfence();
+        if (atomicInc(done + ns, ns - 1) != (unsigned)ns - 1) return;
+        active = atomicExch(&sc->any, 0);
+    }
+    sc->iters = iters + 1;
+    sc->j = J + 1;
+    sc->runs[kBodyInner] = runs + 1;
+    const int go = active && J + 1 < m && iters + 1 < max_iters;
+    sc->flag_inner = go;
+    set_cond(handle, use_h, go);
 }
 
+// V_{j} = w / ||w|| for the next step (j already advanced), while the cycle goes on
 template <typename R>
 __global__ void gm_next_kernel(int64_t nvec, int64_t ldv, const DevScalars* __restrict__ sc,
                                const ShotScalars* __restrict__ ss, const R* __restrict__ w, R* __restrict__ V) {
     constexpr int VW = VL<R>::W;
-    const int J = sc->j;
-    const double hh = ss[blockIdx.y].hcol[J + 1];
-    const R s = (R)(hh > 0.0 ? 1.0 / hh : 0.0);
-    R* vn = V + (int64_t)(J + 1) * ldv;
+    if (!sc->flag_inner || !ss[blockIdx.y].active) return;
+    const R s = (R)ss[blockIdx.y].vscale;
+    R* vn = V + (int64_t)sc->j * ldv;
     seg_loop<R>(nvec,
         [&](int64_t i) {
             R a[VW];
@@ -632,71 +815,41 @@ __global__ void gm_next_kernel(int64_t nvec, int64_t ldv, const DevScalars* __re
         [&](int64_t i) { vn[i] = w[i] * s; });
 }
 
-// Givens update of every shot still iterating; a shot stops at its residual estimate or on
-// breakdown, and keeps the columns it has (jj)
-__global__ void __launch_bounds__(kFinThreads) gm_givens_kernel(DevScalars* sc, ShotScalars* ss, int ns,
-                                                                cudaGraphConditionalHandle h, int use_h) {
-    const int J = sc->j, m = sc->m;
-    int any = 0;
-    for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-        ShotScalars& t = ss[s];
-        if (t.active) {
-            double* hc = t.hcol;
-            for (int i = 0; i < J; ++i) {
-                const double u = t.cs[i] * hc[i] + t.sn[i] * hc[i + 1];
-                hc[i + 1] = -t.sn[i] * hc[i] + t.cs[i] * hc[i + 1];
-                hc[i] = u;
-            }
-            const double a = hc[J], b = hc[J + 1];
-            const double den = hypot(a, b);
-            double cs = 1.0, sn = 0.0;
-            if (den > 0.0) { cs = a / den; sn = b / den; }
-            t.cs[J] = cs;
-            t.sn[J] = sn;
-            hc[J] = den;
-            hc[J + 1] = 0.0;
-            for (int i = 0; i <= J; ++i) t.H[i * kMaxRestart + J] = hc[i];
-            t.g[J + 1] = -sn * t.g[J];
-            t.g[J] = cs * t.g[J];
-            t.resid = fabs(t.g[J + 1]);
-            t.jj = J + 1;
-            if (t.resid <= t.tol_abs || den == 0.0 || !isfinite(t.resid)) t.active = 0;
-        }
-        any |= t.active;
-    }
-    any = __syncthreads_or(any);
-    if (threadIdx.x == 0) {
-        sc->iters += 1;
-        sc->j = J + 1;
-        sc->flag_inner = any && sc->j < m && sc->iters < sc->max_iters;
-        set_cond(h, use_h, sc->flag_inner);
-    }
-}
-
-// y_s = R_s^{-1} g_s (upper triangular, size jj_s)
-__global__ void gm_solve_kernel(ShotScalars* ss, int ns) {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += gridDim.x * blockDim.x) {
-        ShotScalars& t = ss[s];
-        const int J = t.jj;
-        for (int i = J - 1; i >= 0; --i) {
-            double v = t.g[i];
-            for (int k = i + 1; k < J; ++k) v -= t.H[i * kMaxRestart + k] * t.y[k];
-            const double d = t.H[i * kMaxRestart + i];
-            t.y[i] = d != 0.0 ? v / d : 0.0;
+// y = R^{-1} g (upper triangular, size J) of one shot, by every block that needs it: the triangle
+// through shared memory, then one warp eliminates column by column (two unknowns a lane).
+__device__ __forceinline__ void triangular_solve(const ShotScalars& t, int J, double* sH, double* y) {
+    for (int q = threadIdx.x; q < J * J; q += blockDim.x) sH[q] = t.H[(q / J) * kMaxRestart + q % J];
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        double g[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) g[u] = lane + 32 * u < J ? t.g[lane + 32 * u] : 0.0;
+        for (int k = J - 1; k >= 0; --k) {
+            const double d = sH[k * J + k];
+            const double gk = __shfl_sync(0xffffffffu, k < 32 ? g[0] : g[1], k & 31);
+            const double yk = d != 0.0 ? gk / d : 0.0;
+            if (lane == 0) y[k] = yk;
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (lane + 32 * u < k) g[u] -= sH[(lane + 32 * u) * J + k] * yk;
         }
     }
+    __syncthreads();
 }
 
 // x_s += sum_{k<jj_s} y_s[k] V_k  (accumulate = 1), or t_s = sum_k y_s[k] V_k (accumulate = 0;
-// right preconditioning applies P^{-1} to t afterwards)
+// right preconditioning applies P^{-1} to t afterwards), y_s = R_s^{-1} g_s
 template <typename R>
-__global__ void gm_combine_kernel(int64_t nvec, int64_t ldv, const ShotScalars* __restrict__ ss, const R* __restrict__ V,
-                                  R* __restrict__ x, int accumulate) {
+__global__ void __launch_bounds__(256) gm_combine_kernel(int64_t nvec, int64_t ldv, const ShotScalars* __restrict__ ss,
+                                                         const R* __restrict__ V, R* __restrict__ x, int accumulate) {
     constexpr int VW = VL<R>::W;
     const int J = ss[blockIdx.y].jj;
     if (accumulate && J == 0) return;
+    __shared__ double sH[kMaxRestart * kMaxRestart], yd[kMaxRestart];
     __shared__ R y[kMaxRestart];
-    for (int k = threadIdx.x; k < J; k += blockDim.x) y[k] = (R)ss[blockIdx.y].y[k];
+    triangular_solve(ss[blockIdx.y], J, sH, yd);
+    for (int k = threadIdx.x; k < J; k += blockDim.x) y[k] = (R)(-yd[k]);
     __syncthreads();
     seg_loop<R>(nvec,
         [&](int64_t i) {
@@ -706,17 +859,12 @@ __global__ void gm_combine_kernel(int64_t nvec, int64_t ldv, const ShotScalars* 
 #pragma unroll
                 for (int u = 0; u < VW; ++u) a[u] = 0;
             }
-            for (int k = 0; k < J; ++k) {
-                R vv[VW];
-                VL<R>::ld(V + (int64_t)k * ldv + i, vv);
-#pragma unroll
-                for (int u = 0; u < VW; ++u) a[u] = fma(y[k], vv[u], a[u]);
-            }
+            subtract_columns<R, VW>(V, ldv, i, J, y, a);
             VL<R>::st(x + i, a);
         },
         [&](int64_t i) {
             R a = accumulate ? x[i] : (R)0;
-            for (int k = 0; k < J; ++k) a = fma(y[k], V[(int64_t)k * ldv + i], a);
+            for (int k = 0; k < J; ++k) a = fma(-y[k], V[(int64_t)k * ldv + i], a);
             x[i] = a;
         });
 }
@@ -744,6 +892,7 @@ __global__ void __launch_bounds__(kFinThreads) gm_cycle_end_kernel(DevScalars* s
     any = __syncthreads_or(any);
     if (threadIdx.x == 0) {
         sc->j = 0;
+        sc->runs[kBodyCycle] += 1;
         sc->flag_outer = any && sc->iters < sc->max_iters;
         set_cond(h, use_h, sc->flag_outer);
     }
@@ -824,6 +973,7 @@ __global__ void ir_update_kernel(int64_t nvec, const DevScalars* __restrict__ sc
 
 __global__ void ir_end_kernel(DevScalars* sc, cudaGraphConditionalHandle h, int use_h) {
     if (threadIdx.x != 0) return;
+    sc->runs[kBodyIr] += 1;
     if (sc->ir_flag) {
         sc->ir_count += 1;
         sc->st_total += sc->iters;
@@ -857,16 +1007,12 @@ __global__ void __launch_bounds__(kFinThreads) solve_stats_kernel(DevScalars* sc
     } else {
         it = sc->iters;
     }
+    sc->runs[kBodyStraight] += 1;
     if (notconv) sc->st_notconv = 1;
     if (nonfinite) sc->st_nonfinite = 1;
     sc->st_final_rel = rel;
     sc->st_max = max(sc->st_max, it);
     sc->st_iters_sum += (double)it;
-}
-
-// adds a loop body's (or a step's straight-line) kernel count, itself included
-__global__ void count_kernel(DevScalars* sc, long k) {
-    if (threadIdx.x == 0) sc->launches += (unsigned long long)k;
 }
 
 __global__ void step_begin_kernel(double* dparams, double dt) {
@@ -884,10 +1030,11 @@ struct Flow {
     stdg_ctx* c;
     Workspace* ws;
     bool graph;
+    long* kernels;      // kernels of each recorded body
     cudaError_t err = cudaSuccess;
 
-    template <class Init, class Body>
-    void loop(const int* d_flag, Init init, Body body) {
+    template <class Init, class Rec>
+    void loop(Body id, const int* d_flag, Init init, Rec body) {
         if (err != cudaSuccess) return;
         if (!graph) {
             init(cudaGraphConditionalHandle(0), 0);
@@ -896,7 +1043,7 @@ struct Flow {
                 err = cudaMemcpyAsync(&f, d_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
                 if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
                 if (err != cudaSuccess || !f) break;
-                run_body(body, cudaGraphConditionalHandle(0), 0);
+                run_body(id, body, cudaGraphConditionalHandle(0), 0);
             }
             return;
         }
@@ -921,7 +1068,7 @@ struct Flow {
         err = cudaStreamBeginCaptureToGraph(s2, body_g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
         if (err == cudaSuccess) {
             c->stream = s2;
-            run_body(body, h, 1);
+            run_body(id, body, h, 1);
             c->stream = s;
             cudaGraph_t tmp;
             cudaError_t e2 = cudaStreamEndCapture(s2, &tmp);
@@ -932,14 +1079,13 @@ struct Flow {
     }
     void check(cudaError_t e) { if (err == cudaSuccess && e != cudaSuccess) err = e; }
 
-    // one loop body in its own launch-count scope, closed by a count kernel
-    template <class Body>
-    void run_body(Body& body, cudaGraphConditionalHandle h, int use) {
+    // one loop body in its own launch-count scope (the device counts its executions)
+    template <class Rec>
+    void run_body(Body id, Rec& body, cudaGraphConditionalHandle h, int use) {
         c->scopes.push_back(0);
         body(h, use);
-        const long k = c->scopes.back() + 1;
+        kernels[id] = c->scopes.back();
         c->scopes.pop_back();
-        count_kernel<<<1, 32, 0, c->stream>>>(ws->sc, k);
     }
 };
 
@@ -954,24 +1100,23 @@ static void solve_cg(Flow& F, Apply apply, Prec prec, bool use_prec, const R* b,
     const int ns = ws->ns, G = (int)ws->G;
     const dim3 grid = ws->grid();
     R* zz = use_prec ? z : r;
-    F.loop(&ws->sc->flag_inner,
+    F.loop(kBodyInner, &ws->sc->flag_inner,
            [&](cudaGraphConditionalHandle h, int use) {
                F.check(apply(x, q));
                cg_res_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, b, q, r, ws->partials); note_launch(c);
                if (use_prec) F.check(prec(r, zz));
                dot_partial_kernel<R, R><<<grid, kRedThreads, 0, c->stream>>>(nv, r, zz, ws->partials, 2); note_launch(c);
-               cg_init_final_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, rel_tol, max_iters,
+               cg_init_final_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, rel_tol, max_iters,
                                                                       bnorm_given, gate_ir, h, use); note_launch(c);
                copy_kernel<R><<<ws->red_blocks, kRedThreads, 0, c->stream>>>(n, zz, p); note_launch(c);
            },
            [&](cudaGraphConditionalHandle h, int use) {
                F.check(apply(p, q));
-               dot_partial_kernel<R, R><<<grid, kRedThreads, 0, c->stream>>>(nv, p, q, ws->partials, 0); note_launch(c);
-               cg_alpha_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->ss, ws->partials, ns, G); note_launch(c);
+               cg_dot_alpha_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, p, q, ws->partials, ws->ss, ws->done); note_launch(c);
                cg_update_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ws->ss, x, r, p, q, ws->partials); note_launch(c);
                if (use_prec) F.check(prec(r, zz));
-               dot_partial_kernel<R, R><<<grid, kRedThreads, 0, c->stream>>>(nv, r, zz, ws->partials, 2); note_launch(c);
-               cg_beta_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, h, use); note_launch(c);
+               cg_dot_beta_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, r, zz, ws->partials, ws->sc, ws->ss, ws->done, h,
+                                                                          use); note_launch(c);
                cg_p_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ws->ss, zz, p); note_launch(c);
                F.check(cudaGetLastError());
            });
@@ -990,21 +1135,23 @@ static void solve_gmres(Flow& F, Apply apply, ApplyIdx apply_idx, Prec prec, boo
     DevScalars* sc = ws->sc;
     ShotScalars* ss = ws->ss;
     double* part = ws->partials;
-    F.loop(&sc->flag_outer,
+    const dim3 dot_grid = ws->dot_grid();
+    unsigned* done = ws->done;
+    F.loop(kBodyCycle, &sc->flag_outer,
            [&](cudaGraphConditionalHandle h, int use) {
                if (bnorm_given < 0) {
                    dot_partial_kernel<R, R><<<grid, kRedThreads, 0, c->stream>>>(nv, b, b, part, 0); note_launch(c);
                }
-               gm_init_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, part, ns, G, rel_tol, max_iters, m, bnorm_given,
-                                                                gate_ir, h, use); note_launch(c);
+               gm_init_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(sc, ss, part, ns, G, rel_tol, max_iters, m, bnorm_given,
+                                                                      gate_ir, h, use); note_launch(c);
            },
            [&](cudaGraphConditionalHandle h_outer, int use_outer) {
                // restart cycle: true residual, then Arnoldi
                F.check(apply(x, w));
-               gm_res_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, b, w, V, part); note_launch(c);
-               F.loop(&sc->flag_inner,
+               F.loop(kBodyInner, &sc->flag_inner,
                       [&](cudaGraphConditionalHandle h, int use) {
-                          gm_cycle_start_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, part, ns, G, h, use); note_launch(c);
+                          gm_res_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, b, w, V, part, 1, sc, ss, done, h, use);
+                          note_launch(c);
                           gm_scale0_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, sc, ss, V); note_launch(c);
                       },
                       [&](cudaGraphConditionalHandle h, int use) {
@@ -1015,18 +1162,17 @@ static void solve_gmres(Flow& F, Apply apply, ApplyIdx apply_idx, Prec prec, boo
                               F.check(apply_idx(V, &sc->j, w));
                           }
                           // classical Gram-Schmidt: dots and ||w||^2; a second pass (with the first
-                          // subtraction fused in) only for the shots that need it; subtraction + norm
-                          gm_mdot_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, V, w, part); note_launch(c);
-                          gm_mdot_final_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, part, ns, G, 0); note_launch(c);
-                          gm_orth_fused_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, ss, V, w, part); note_launch(c);
-                          gm_mdot_final_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, part, ns, G, 1); note_launch(c);
-                          gm_maxpy_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, ss, V, w, part); note_launch(c);
-                          gm_norm_final_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, part, ns, G); note_launch(c);
+                          // subtraction fused in) only for the shots that need it; subtraction, norm,
+                          // Givens rotations and loop control
+                          gm_mdot_kernel<R><<<dot_grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, ss, V, w, part, done);
+                          note_launch(c);
+                          gm_orth_fused_kernel<R><<<dot_grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, ss, V, w, part, done);
+                          note_launch(c);
+                          gm_maxpy_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, ss, V, w, part, done, h, use);
+                          note_launch(c);
                           gm_next_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, sc, ss, w, V); note_launch(c);
-                          gm_givens_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, ns, h, use); note_launch(c);
                           F.check(cudaGetLastError());
                       });
-               gm_solve_kernel<<<(ns + 127) / 128, 128, 0, c->stream>>>(ss, ns); note_launch(c);
                if (use_prec) {   // x += P^{-1} (V y)
                    gm_combine_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, ss, V, tbuf, 0); note_launch(c);
                    F.check(prec(tbuf, zbuf, nullptr, 0));
@@ -1034,7 +1180,7 @@ static void solve_gmres(Flow& F, Apply apply, ApplyIdx apply_idx, Prec prec, boo
                } else {
                    gm_combine_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ldv, ss, V, x, 1); note_launch(c);
                }
-               gm_cycle_end_kernel<<<1, kFinThreads, 0, c->stream>>>(sc, ss, ns, h_outer, use_outer); note_launch(c);
+               gm_cycle_end_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(sc, ss, ns, h_outer, use_outer); note_launch(c);
                F.check(cudaGetLastError());
            });
 }
@@ -1069,19 +1215,20 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
         if (cn) solve_cg<double>(F, A64, P64c, pre, b, x, ws->r, ws->p, ws->q, ws->z, tol, maxit, -1.0, 0);
         else solve_gmres<double>(F, A64, A64i, P64, pre, b, x, ws->V, ws->w, ws->z, ws->t, tol, maxit, -1.0, 0);
         zero_if_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, x, ws->ss, 0); note_launch(c);
-        solve_stats_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->sc, ws->ss, ns, cn ? 1 : 0); note_launch(c);
+        solve_stats_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ns, cn ? 1 : 0); note_launch(c);
         return;
     }
     // mixed: FP64 refinement, FP32 inner solve with zero initial guess and unit RHS per shot
-    F.loop(&ws->sc->ir_flag,
+    F.loop(kBodyIr, &ws->sc->ir_flag,
            [&](cudaGraphConditionalHandle h, int use) {
                dot_partial_kernel<double, double><<<grid, kRedThreads, 0, c->stream>>>(nv, b, b, ws->partials, 0); note_launch(c);
-               ir_init_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, tol, 64, h, use); note_launch(c);
+               ir_init_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, tol, 64, h, use); note_launch(c);
            },
            [&](cudaGraphConditionalHandle h, int use) {
                F.check(A64(x, ws->w));
-               gm_res_kernel<double><<<grid, kRedThreads, 0, c->stream>>>(nv, b, ws->w, ws->r, ws->partials); note_launch(c);
-               ir_check_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, maxit); note_launch(c);
+               gm_res_kernel<double><<<grid, kRedThreads, 0, c->stream>>>(nv, b, ws->w, ws->r, ws->partials, 0, ws->sc, ws->ss,
+                                                                          ws->done, 0, 0); note_launch(c);
+               ir_check_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, maxit); note_launch(c);
                ir_convert_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, ws->sc, ws->ss, ws->r, ws->b32, ws->x32); note_launch(c);
                if (cn)
                    solve_cg<float>(F, A32, P32c, pre, ws->b32, ws->x32, ws->r32, ws->p32, ws->q32, ws->z32, c->opt.inner_tol,
@@ -1094,7 +1241,7 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
                F.check(cudaGetLastError());
            });
     zero_if_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, x, ws->ss, 1); note_launch(c);
-    solve_stats_kernel<<<1, kFinThreads, 0, c->stream>>>(ws->sc, ws->ss, ns, 2); note_launch(c);
+    solve_stats_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ns, 2); note_launch(c);
 }
 
 // One slab for every shot: per-shot right-hand sides and initial guesses, ONE stacked
@@ -1116,9 +1263,8 @@ static void record_step(Flow& F, double dt) {
         F.check(launch_receivers(c, ws->dparams, shot));
     }
     step_end_kernel<<<1, 32, 0, c->stream>>>(ws->dparams, dt); note_launch(c);
-    const long k = c->scopes.back() + 1;
+    F.kernels[kBodyStraight] = c->scopes.back();
     c->scopes.clear();
-    count_kernel<<<1, 32, 0, c->stream>>>(ws->sc, k);
     F.check(cudaGetLastError());
 }
 
@@ -1130,9 +1276,18 @@ int solver_setup(stdg_ctx* c) {
     ws->ns = c->n_shots;
     ws->nvec = c->nvel;
     ws->n = c->nvel * (int64_t)c->n_shots;
-    ws->red_blocks = (unsigned)(8 * c->n_sm);
-    ws->G = (unsigned)std::max(1, (int)ws->red_blocks / ws->ns);
+    // Grids by vector length: one 16-byte item a thread, up to the blocks that keep every SM busy.
+    // (A fixed grid made every launch on a 2,352-value vector start 1,216 blocks and every reduction
+    // sum as many parts: 49 us per CG iteration.)
+    const int64_t item = c->opt.precision == STDG_FP64 ? 2 : 4;
+    auto blocks = [&](int64_t values, int per_sm, int shots) {
+        const int64_t want = (values + item * kRedThreads - 1) / (item * kRedThreads);
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)per_sm * c->n_sm / shots));
+    };
     const int64_t n = ws->n;
+    ws->red_blocks = blocks(n, 8, 1);
+    ws->G = blocks(ws->nvec, 4, ws->ns);
+    ws->Gd = blocks(ws->nvec, 2, ws->ns);
     const bool cn = c->opt.scheme == STDG_SCHEME_CN && c->opt.preconditioner != 2;   // CG workspace
     const bool mixed = c->opt.precision != STDG_FP64;
     const bool pre = c->opt.preconditioner != 0;
@@ -1142,6 +1297,7 @@ int solver_setup(stdg_ctx* c) {
     ALLOC(ws->sc, sizeof(DevScalars));
     ALLOC(ws->ss, sizeof(ShotScalars) * ws->ns);
     ALLOC(ws->partials, sizeof(double) * (kMaxRestart + 2) * ws->G * ws->ns);
+    ALLOC(ws->done, sizeof(unsigned) * (ws->ns + 1));
     ALLOC(ws->dparams, sizeof(double) * 4);
     ALLOC(c->d_b, sizeof(double) * n);
     ALLOC(c->d_x, sizeof(double) * n);
@@ -1161,6 +1317,7 @@ int solver_setup(stdg_ctx* c) {
 #undef ALLOC
     cudaMemsetAsync(ws->sc, 0, sizeof(DevScalars), c->stream);
     cudaMemsetAsync(ws->ss, 0, sizeof(ShotScalars) * ws->ns, c->stream);
+    cudaMemsetAsync(ws->done, 0, sizeof(unsigned) * (ws->ns + 1), c->stream);
     cudaMemsetAsync(ws->dparams, 0, sizeof(double) * 4, c->stream);
     for (auto& s : ws->side) cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
     return STDG_OK;
@@ -1200,9 +1357,8 @@ static void record_solve_only(Flow& F, double dt) {
     stdg_ctx* c = F.c;
     c->scopes.assign(1, 0);
     record_solve(F, dt, c->d_b, c->d_x);
-    const long k = c->scopes.back() + 1;
+    F.kernels[kBodyStraight] = c->scopes.back();
     c->scopes.clear();
-    count_kernel<<<1, 32, 0, c->stream>>>(F.ws->sc, k);
     F.check(cudaGetLastError());
 }
 
@@ -1212,7 +1368,7 @@ static int run_body_n(stdg_ctx* c, double dt, int n, int kind, stdg_stats* st) {
     Workspace* ws = W(c);
     STDG_CUDA(c, cudaMemsetAsync(&ws->sc->st_total, 0, sizeof(int) * 5, c->stream));
     STDG_CUDA(c, cudaMemsetAsync(&ws->sc->st_final_rel, 0, sizeof(double) * 2, c->stream));
-    STDG_CUDA(c, cudaMemsetAsync(&ws->sc->launches, 0, sizeof(unsigned long long), c->stream));
+    STDG_CUDA(c, cudaMemsetAsync(ws->sc->runs, 0, sizeof(ws->sc->runs), c->stream));
     auto record = [&](Flow& F) {
         if (kind == 0) record_step(F, dt);
         else record_solve_only(F, dt);
@@ -1225,7 +1381,7 @@ static int run_body_n(stdg_ctx* c, double dt, int n, int kind, stdg_stats* st) {
             ws->graph[kind] = nullptr;
             cudaStream_t s0 = c->stream;
             STDG_CUDA(c, cudaStreamBeginCapture(s0, cudaStreamCaptureModeRelaxed));
-            Flow F{c, ws, true};
+            Flow F{c, ws, true, ws->body_kernels[kind]};
             record(F);
             c->stream = s0;
             cudaGraph_t g = nullptr;
@@ -1243,7 +1399,7 @@ static int run_body_n(stdg_ctx* c, double dt, int n, int kind, stdg_stats* st) {
         for (int s = 0; s < n; ++s) STDG_CUDA(c, cudaGraphLaunch(ws->exec[kind], c->stream));
     } else {
         for (int s = 0; s < n; ++s) {
-            Flow F{c, ws, false};
+            Flow F{c, ws, false, ws->body_kernels[kind]};
             record(F);
             if (F.err != cudaSuccess) STDG_CUDA(c, F.err);
         }
@@ -1259,7 +1415,8 @@ static int run_body_n(stdg_ctx* c, double dt, int n, int kind, stdg_stats* st) {
         st->final_rel_res = h.st_final_rel;
         st->status = h.st_nonfinite ? STDG_ENONFINITE : h.st_notconv ? STDG_ENOTCONV : STDG_OK;
     }
-    c->last_launches = (int64_t)h.launches;
+    c->last_launches = 0;
+    for (int i = 0; i < kBodies; ++i) c->last_launches += (int64_t)h.runs[i] * ws->body_kernels[kind][i];
     {
         const int rc = take_device_error(c);
         if (rc != STDG_OK) return rc;
