@@ -10,10 +10,24 @@ namespace stdg {
 void solver_invalidate_graph(stdg_ctx* c);
 double* solver_dparams(stdg_ctx* c);
 
+// Gives the assembled couplings back; captured graphs may hold their addresses.
+static void drop_coupling(stdg_ctx* c) {
+    solver_invalidate_graph(c);
+    cudaStreamSynchronize(c->stream);
+    for (void* p : {(void*)c->d_Kf, (void*)c->d_Ke, (void*)c->d_Kf32, (void*)c->d_Ke32}) dev_release(c, p);
+    c->d_Kf = c->d_Ke = nullptr;
+    c->d_Kf32 = c->d_Ke32 = nullptr;
+}
+
 int dev_alloc(stdg_ctx* c, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && c->d_Kf) {   // the couplings only save time: everything else comes first
+        cudaGetLastError();
+        drop_coupling(c);
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         c->err = std::string("cudaMalloc(") + std::to_string(bytes) + "): " + cudaGetErrorString(e);
@@ -151,6 +165,43 @@ static int ensure_fp32(stdg_ctx* c) {
     return STDG_OK;
 }
 
+// Assembled couplings of the current medium (FP64, and their FP32 copy where D~ has one).  They are
+// left out where they would take more than a third of the free memory.
+static int setup_coupling(stdg_ctx* c) {
+    const int64_t n2 = (int64_t)c->dim * c->Nphi * c->dim * c->Nphi, nKf = c->n_face * n2, nKe = c->n_elem * n2;
+    const bool want32 = c->d_D32 != nullptr && coupling32_wanted(c);
+    if (!c->d_Kf) {
+        size_t free_b = 0, total_b = 0;
+        STDG_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
+        if ((size_t)(nKf + nKe) * (want32 ? 16 : 8) > free_b / 3) return STDG_OK;
+        double *kf = nullptr, *ke = nullptr;
+        if (dev_alloc(c, (void**)&kf, sizeof(double) * nKf) != STDG_OK || dev_alloc(c, (void**)&ke, sizeof(double) * nKe) != STDG_OK) {
+            dev_release(c, kf);
+            return STDG_OK;
+        }
+        c->d_Kf = kf;
+        c->d_Ke = ke;
+    }
+    STDG_CUDA(c, launch_coupling_setup(c));
+    if (!want32) return STDG_OK;
+    if (!c->d_Kf32) {
+        float *kf = nullptr, *ke = nullptr;
+        if (dev_alloc(c, (void**)&kf, sizeof(float) * 2 * nKf) != STDG_OK || dev_alloc(c, (void**)&ke, sizeof(float) * nKe) != STDG_OK) {
+            dev_release(c, kf);
+            return STDG_OK;
+        }
+        if (!c->d_Kf) {   // dropped to make room for these: the FP32 copy alone is of no use
+            dev_release(c, kf);
+            dev_release(c, ke);
+            return STDG_OK;
+        }
+        c->d_Kf32 = kf;
+        c->d_Ke32 = ke;
+    }
+    STDG_CUDA(c, launch_coupling_cast(c));
+    return STDG_OK;
+}
+
 static int upload_material32(stdg_ctx* c) {
     if (!c->have_material || !c->d_D32) return STDG_OK;
     std::vector<float> lf(c->n_face), mf(c->n_face), rj(c->n_elem);
@@ -199,7 +250,6 @@ static int setup_pre1(stdg_ctx* c) {
     if (status) STDG_FAIL(c, STDG_ECUDA, "block-Jacobi eigen-decomposition did not converge");
     if (c->d_preV32) {
         const int64_t nv = ne * n * n;
-        extern cudaError_t launch_cast32(stdg_ctx*, const double*, float*, int64_t);
         STDG_CUDA(c, launch_cast32(c, c->d_preV, c->d_preV32, nv));
     }
     if (c->opt.preconditioner == 2) {
@@ -378,6 +428,9 @@ int stdg_set_mesh(stdg_ctx* c, int64_t n_vert, const double* xyz, int64_t n_elem
     c->d_preV = c->d_preLam = c->d_preB = nullptr;
     c->d_preV32 = c->d_preB32 = nullptr;
     c->d_preB32t = nullptr;
+    c->d_Kf = c->d_Ke = nullptr;
+    c->d_Kf32 = c->d_Ke32 = nullptr;
+    c->d_adj = nullptr;
     c->d_pre2 = nullptr;
     c->d_pre2_32 = nullptr;
     c->d_pre2_mma = nullptr;
@@ -442,6 +495,15 @@ int stdg_set_mesh(stdg_ctx* c, int64_t n_vert, const double* xyz, int64_t n_elem
     UP(c->d_face_l, c->hm.face_l.data(), sizeof(int32_t) * nf);
     UP(c->d_elem_face, c->hm.elem_face.data(), sizeof(int32_t) * n_elem * nv);
     UP(c->d_face_r, c->hm.face_r.data(), sizeof(int32_t) * nf);
+    {
+        std::vector<int2> adj((size_t)n_elem * nv);
+        for (int64_t q = 0; q < n_elem * nv; ++q) {
+            const int32_t e = (int32_t)(q / nv), f = c->hm.elem_face[q], l = c->hm.face_l[f];
+            adj[q] = l == e ? make_int2(c->hm.face_r[f], 2 * f) : make_int2(l, 2 * f + 1);
+        }
+        ALLOC(c->d_adj, sizeof(int2) * adj.size());
+        UP(c->d_adj, adj.data(), sizeof(int2) * adj.size());
+    }
     UP(c->d_X, c->hm.X.data(), sizeof(double) * n_elem * nv * d);
     UP(c->d_Jinv, c->hm.Jinv.data(), sizeof(double) * n_elem * d * d);
     UP(c->d_detJ, c->hm.detJ.data(), sizeof(double) * n_elem);
@@ -546,6 +608,7 @@ static int upload_material(stdg_ctx* c) {
     c->have_material = true;
     rc = upload_material32(c);
     if (rc != STDG_OK) return rc;
+    if ((rc = setup_coupling(c)) != STDG_OK) return rc;
     if (c->opt.preconditioner) return setup_pre1(c);
     return STDG_OK;
 }

@@ -433,8 +433,7 @@ cudaError_t launch_pre2_local_batch(stdg_ctx* c, const float* r, const float* w,
 }
 
 // z = P_2 r for nshots stacked shots: y = P_1 r, w = A y, z = S^{-1} (2 r - w).
-// Since D_i y_i = r_i, (2 r - A y)_i = r_i - sum_e N_{i,e} y_e: the neighbour coupling comes
-// out of one ordinary operator application.
+// Since D_i y_i = r_i, A y = r + sum_e N_{i,e} y_e: only the neighbour couplings are applied.
 template <typename R, typename S>
 static cudaError_t pre2_apply_t(stdg_ctx* c, const S* Sinv, int64_t es, const R* r, R* z, const int* ridx, int64_t ld,
                                 int nshots, bool fp32) {
@@ -443,10 +442,12 @@ static cudaError_t pre2_apply_t(stdg_ctx* c, const S* Sinv, int64_t es, const R*
     cudaError_t e;
     if (fp32) {
         if ((e = launch_pre1_apply32(c, (const float*)r, (float*)y, ridx, ld, nshots)) != cudaSuccess) return e;
-        if ((e = launch_apply32(c, c->pre_dt, (const float*)y, (float*)w, 1.0, nullptr, 0, nshots)) != cudaSuccess) return e;
+        if ((e = launch_apply_pre1_32(c, c->pre_dt, (const float*)y, (const float*)r, ridx, ld, (float*)w, nshots)) != cudaSuccess)
+            return e;
     } else {
         if ((e = launch_pre1_apply(c, (const double*)r, (double*)y, ridx, ld, nshots)) != cudaSuccess) return e;
-        if ((e = launch_apply(c, c->pre_dt, (const double*)y, (double*)w, 1.0, nullptr, 0, nshots)) != cudaSuccess) return e;
+        if ((e = launch_apply_pre1(c, c->pre_dt, (const double*)y, (const double*)r, ridx, ld, (double*)w, nshots)) != cudaSuccess)
+            return e;
     }
     return pre2_local_t<R, S>(c, Sinv, es, r, ridx, ld, w, z, nshots);
 }

@@ -1123,8 +1123,10 @@ static void solve_cg(Flow& F, Apply apply, Prec prec, bool use_prec, const R* b,
 }
 
 // ---- GMRES(m) on vectors of type R -----------------------------------------------------
-template <typename R, class Apply, class ApplyIdx, class Prec>
-static void solve_gmres(Flow& F, Apply apply, ApplyIdx apply_idx, Prec prec, bool use_prec, const R* b, R* x, R* V, R* w,
+// apply_prec(z, V, j, ld, w): w = A z for z = prec(V_j)
+template <typename R, class Apply, class ApplyIdx, class ApplyPrec, class Prec>
+static void solve_gmres(Flow& F, Apply apply, ApplyIdx apply_idx, ApplyPrec apply_prec, Prec prec, bool use_prec, const R* b,
+                        R* x, R* V, R* w,
                         R* zbuf, R* tbuf, double rel_tol, int max_iters, double bnorm_given, int gate_ir) {
     stdg_ctx* c = F.c;
     Workspace* ws = F.ws;
@@ -1157,7 +1159,7 @@ static void solve_gmres(Flow& F, Apply apply, ApplyIdx apply_idx, Prec prec, boo
                       [&](cudaGraphConditionalHandle h, int use) {
                           if (use_prec) {   // right preconditioning: w = A P^{-1} v_j
                               F.check(prec(V, zbuf, &sc->j, ldv));
-                              F.check(apply(zbuf, w));
+                              F.check(apply_prec(zbuf, V, &sc->j, ldv, w));
                           } else {
                               F.check(apply_idx(V, &sc->j, w));
                           }
@@ -1201,6 +1203,12 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
     auto A64i = [&](const double* V, const int* idx, double* yy) { return launch_apply(c, dt, V, yy, 1.0, idx, ldv, ns); };
     auto A32 = [&](const float* xx, float* yy) { return launch_apply32(c, dt, xx, yy, 1.0, nullptr, 0, ns); };
     auto A32i = [&](const float* V, const int* idx, float* yy) { return launch_apply32(c, dt, V, yy, 1.0, idx, ldv, ns); };
+    auto AP64 = [&](const double* z, const double* V, const int* idx, int64_t ld, double* w) {
+        return p2 ? launch_apply(c, dt, z, w, 1.0, nullptr, 0, ns) : launch_apply_pre1(c, dt, z, V, idx, ld, w, ns);
+    };
+    auto AP32 = [&](const float* z, const float* V, const int* idx, int64_t ld, float* w) {
+        return p2 ? launch_apply32(c, dt, z, w, 1.0, nullptr, 0, ns) : launch_apply_pre1_32(c, dt, z, V, idx, ld, w, ns);
+    };
     auto P64 = [&](const double* r, double* z, const int* idx, int64_t ld) {
         return p2 ? launch_pre2_apply(c, r, z, idx, ld, ns) : launch_pre1_apply(c, r, z, idx, ld, ns);
     };
@@ -1213,7 +1221,7 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
     const int maxit = c->opt.max_iters;
     if (c->opt.precision == STDG_FP64) {
         if (cn) solve_cg<double>(F, A64, P64c, pre, b, x, ws->r, ws->p, ws->q, ws->z, tol, maxit, -1.0, 0);
-        else solve_gmres<double>(F, A64, A64i, P64, pre, b, x, ws->V, ws->w, ws->z, ws->t, tol, maxit, -1.0, 0);
+        else solve_gmres<double>(F, A64, A64i, AP64, P64, pre, b, x, ws->V, ws->w, ws->z, ws->t, tol, maxit, -1.0, 0);
         zero_if_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, x, ws->ss, 0); note_launch(c);
         solve_stats_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ns, cn ? 1 : 0); note_launch(c);
         return;
@@ -1234,7 +1242,7 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
                    solve_cg<float>(F, A32, P32c, pre, ws->b32, ws->x32, ws->r32, ws->p32, ws->q32, ws->z32, c->opt.inner_tol,
                                    maxit, 1.0, 1);
                else
-                   solve_gmres<float>(F, A32, A32i, P32, pre, ws->b32, ws->x32, ws->V32, ws->w32, ws->z32, ws->t32,
+                   solve_gmres<float>(F, A32, A32i, AP32, P32, pre, ws->b32, ws->x32, ws->V32, ws->w32, ws->z32, ws->t32,
                                       c->opt.inner_tol, maxit, 1.0, 1);
                ir_update_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, ws->sc, ws->ss, ws->x32, x); note_launch(c);
                ir_end_kernel<<<1, 32, 0, c->stream>>>(ws->sc, h, use); note_launch(c);

@@ -120,6 +120,12 @@ struct stdg_ctx {
     double *d_lamf_ph = nullptr, *d_muf_ph = nullptr, *d_rhoJ_ph = nullptr;
     std::vector<double> alpha_e;       // per-element time scale; empty: 1 everywhere
     float *d_lamf32 = nullptr, *d_muf32 = nullptr, *d_rhoJ32 = nullptr;
+    // assembled couplings of the operator (coupling.cu): K_lr per face, K_ii per element, rows and
+    // columns (k, n); null when the device cannot hold them (the face kernels then apply D~).  The FP32
+    // copy has the faces' blocks in both orientations
+    double *d_Kf = nullptr, *d_Ke = nullptr;
+    float *d_Kf32 = nullptr, *d_Ke32 = nullptr;
+    int2* d_adj = nullptr;      // [e][dim + 1]: neighbour (-1 on the boundary), 2 face + side of e
 
     // ---- device: state (shot-major)
     double *d_vtr = nullptr, *d_sigtr = nullptr;
@@ -219,6 +225,12 @@ cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, dou
                          const int* xidx = nullptr, int64_t ld = 0, int nshots = 1);
 cudaError_t launch_apply32(stdg_ctx* c, double dt, const float* x, float* y, double cfac,
                            const int* xidx = nullptr, int64_t ld = 0, int nshots = 1);
+// w = A y for y = P_1 base (the exact block-Jacobi inverse, so D y = base): base plus the off-diagonal
+// couplings of y where the assembled couplings are kept, one ordinary application otherwise
+cudaError_t launch_apply_pre1(stdg_ctx* c, double dt, const double* y, const double* base, const int* bidx, int64_t bld,
+                              double* w, int nshots);
+cudaError_t launch_apply_pre1_32(stdg_ctx* c, double dt, const float* y, const float* base, const int* bidx, int64_t bld,
+                                 float* w, int nshots);
 cudaError_t launch_face_only(stdg_ctx* c, double dt, const void* x, void* y, double cfac, int fp32);
 cudaError_t launch_rhs(stdg_ctx* c, double dt, const double* dparams, int shot, double* b);
 cudaError_t launch_stress_update(stdg_ctx* c, double dt, int shot, const double* x);
@@ -233,6 +245,17 @@ cudaError_t launch_initial_guess(stdg_ctx* c, int shot, double* x);
 template <typename R>
 bool launch_face_fast(stdg_ctx* c, const R* D, const R* lamf, const R* muf, const R* x, const int* xidx, int64_t ld, R* y,
                       double scale, cudaError_t* err, int nshots = 1);
+
+// coupling.cu: the operator from its assembled couplings; base == null: y = A x with `scale` on the
+// Schur part; otherwise y = base + scale (off-diagonal Schur part of x)
+cudaError_t launch_coupling_setup(stdg_ctx* c);
+cudaError_t launch_coupling_cast(stdg_ctx* c);
+cudaError_t launch_cast32(stdg_ctx* c, const double* a, float* b, int64_t n);   // kernels.cu
+bool coupling32_wanted(const stdg_ctx* c);   // whether this shape's FP32 operator uses them (kernels.cu)
+cudaError_t launch_coupling(stdg_ctx* c, const double* x, const int* xidx, int64_t ld, const double* base, const int* bidx,
+                            int64_t bld, double* y, double scale, int nshots);
+cudaError_t launch_coupling32(stdg_ctx* c, const float* x, const int* xidx, int64_t ld, const float* base, const int* bidx,
+                              int64_t bld, float* y, double scale, int nshots);
 
 // precond.cu
 cudaError_t launch_pre1_setup(stdg_ctx* c, const double* d_Rinv, const int32_t* d_elem_face, int* d_status);

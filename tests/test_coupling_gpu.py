@@ -1,0 +1,97 @@
+"""The operator from assembled couplings (csrc/coupling*.cu) over every order it is instantiated for,
+against the assembled oracle; the off-diagonal form inside the stencil preconditioner for shot counts
+around the four that a thread carries; and the face kernels when the couplings do not fit the device.
+Bars: 1e-12 in FP64 and 2e-5 in FP32 for the operator (as the other operator tests), 1e-9 / 1e-3 for
+the preconditioner (FP64; FP32 with 16-bit or TF32 blocks)."""
+import numpy as np
+import pytest
+
+import synth
+from helpers import extended_patch_rows, need_gpu, oracle_sim, rel_l2, rel_l2_ext
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(2, p, pg) for p in (1, 2, 3, 4) for pg in range(5)] + [(3, p, pg) for p in (1, 2, 3) for pg in (0, 1, 3)] + \
+    [(3, 2, 2), (3, 1, 4)]
+
+
+def _workload(dim, p, pg, n=2):
+    if dim == 2:
+        xyz, ev, per = synth.tri_grid(n + 1, n, 1.0, 1.0, periodic=False, jitter=0.2, seed=3)
+    else:
+        xyz, ev, per = synth.tet_kuhn(1 if p == 3 else 2, 1.0, periodic=False, jitter=0.1, seed=3)
+    ne = ev.shape[0]
+    rng = np.random.default_rng(5)
+    return synth.Workload("coupling", dim, xyz, ev, per, rng.uniform(1, 2, ne), rng.uniform(.5, 1, ne),
+                          rng.uniform(.8, 1.2, ne), p=p, p_gamma=pg, scheme="stdg", dt=0.05, n_steps=1, h=1.0 / n)
+
+
+def _solver(w, **kw):
+    from paper_1802_04516_gb300.binding import Solver
+    s = Solver(w.dim, w.p, w.p_gamma, scheme=w.scheme, **kw)
+    s.set_mesh(w.xyz, w.elem_vert, w.period)
+    s.set_material(w.lam, w.mu, w.rho)
+    return s
+
+
+@pytest.mark.parametrize("dim,p,pg", SHAPES)
+def test_operator_of_every_order(dim, p, pg):
+    torch = need_gpu()
+    w = _workload(dim, p, pg)
+    A = oracle_sim(w).A
+    s = _solver(w, precision="mixed", preconditioner=0)
+    x = np.random.default_rng(6).normal(size=A.shape[0])
+    ref = A @ x
+    y = s.apply_operator(w.dt, x)
+    if p == 4:   # the FP64 oracle's own rounding is above the bar there: every row in extended precision
+        elems = list(range(w.n_elem))
+        assert rel_l2_ext(y.reshape(w.n_elem, -1), extended_patch_rows(w, elems, x)) < 1e-12
+    else:
+        assert rel_l2(y, ref) < 1e-12
+    xd = torch.tensor(x, dtype=torch.float32, device="cuda")
+    yd = torch.zeros_like(xd)
+    torch.cuda.synchronize()
+    s.apply_operator_device(w.dt, xd.data_ptr(), yd.data_ptr(), fp32=True)
+    assert rel_l2(yd.double().cpu().numpy(), ref) < 2e-5
+
+
+@pytest.mark.parametrize("dim,p,pg,shots", [(2, 1, 1, 3), (2, 2, 2, 4), (2, 2, 2, 29), (2, 3, 2, 5), (2, 3, 3, 2), (3, 1, 1, 6),
+                                            (3, 2, 1, 1)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_off_diagonal_form_for_stacked_shots(dim, p, pg, shots, precision):
+    torch = need_gpu()
+    from oracle.precond import pre2
+    w = _workload(dim, p, pg)
+    sim = oracle_sim(w)
+    P = pre2(sim.A, w.n_elem, sim.mesh.elem_nbr)
+    s = _solver(w, precision=precision, preconditioner=2)
+    s.set_shots(shots)
+    r = np.random.default_rng(7).normal(size=(shots, sim.A.shape[0]))
+    dtype = torch.float64 if precision == "fp64" else torch.float32
+    rd = torch.tensor(r, dtype=dtype, device="cuda")
+    zd = torch.zeros_like(rd)
+    torch.cuda.synchronize()
+    s.apply_preconditioner_device(w.dt, rd.data_ptr(), zd.data_ptr(), fp32=precision == "mixed")
+    z = zd.double().cpu().numpy()
+    for k in range(shots):
+        assert rel_l2(z[k], P @ r[k]) < (1e-9 if precision == "fp64" else 1e-3)
+
+
+def test_face_kernels_when_the_couplings_do_not_fit():
+    torch = need_gpu()
+    w = _workload(2, 3, 3, n=60)
+    x = np.random.default_rng(8).normal(size=w.n_elem * 2 * 4 * 10)
+    s = _solver(w, preconditioner=1)
+    y, held = s.apply_operator(w.dt, x), s.query(10)
+    s.close()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    fill = torch.empty(free - (held - (16 << 20)), dtype=torch.uint8, device="cuda")   # room for all but the couplings
+    try:
+        s = _solver(w, preconditioner=1)
+        assert s.query(10) < held
+        assert rel_l2(s.apply_operator(w.dt, x), y) < 1e-12
+    finally:
+        s.close()
+        del fill
+        torch.cuda.empty_cache()
