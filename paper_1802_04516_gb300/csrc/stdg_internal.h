@@ -93,6 +93,7 @@ struct stdg_ctx {
     bool own_stream = false;
     std::string err;
     bool have_mesh = false, have_material = false;
+    bool material32 = false;     // the FP32 copies of the material are those of the current one
 
     stdg::RefTables rt{};
     stdg::HostMesh hm;
@@ -170,6 +171,7 @@ struct stdg_ctx {
     // arrive in time; 2: a copy still in flight could not be drained).  Read and cleared by
     // take_device_error after every call that can launch such a kernel.
     int* d_err = nullptr;
+    int* h_err = nullptr;        // pinned copy of the word, read after a synchronisation of the stream
     bool wait_gave_up = false;   // the last take_device_error found the word set
     bool echeck_on = false;      // energy-growth sentinel around stdg_step
     double echeck_tol = 0.0;
