@@ -163,6 +163,8 @@ cudaError_t launch_coupling(stdg_ctx* c, const double* x, const int* xidx, int64
 }
 cudaError_t launch_coupling32(stdg_ctx* c, const float* x, const int* xidx, int64_t ld, const float* base, const int* bidx,
                               int64_t bld, float* y, double scale, int nshots) {
+    if (coupling_shots_applies(c, nshots, x, ld, base, bld, y))
+        return launch_coupling_shots(c, x, xidx, ld, base, bidx, bld, y, scale, nshots);
     auto go = c->dim == 2 ? coupling_2d<float> : coupling_3d<float>;
     return go(c, c->d_Ke32, c->d_Kf32, c->d_rhoJ32, x, xidx, ld, base, bidx, bld, y, scale, nshots);
 }

@@ -736,19 +736,13 @@ cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, dou
 // against 310 us with the mass term on 82,944 tetrahedra), and 2D at p = p_gamma = 3, where they are
 // faster (264 against 325 us on 200,704 triangles) but move the mixed slab of the sliver mesh by more
 // than two runs differ (its inner residual is met by a different iterate; single velocities by 3e-7).
-// Elsewhere they win for one shot at every size (2D p = 2: 117 against 238 us on 200,704 triangles)
-// and for a few shots; from 16 shots (28 for the off-diagonal part alone) the kernel with one lane per
-// shot, which reads a face's block once for 32 shots, is faster (64 shots on 12,544 triangles: 374
-// against 280 us).
+// Elsewhere they win at every size (2D p = 2: 117 against 238 us on 200,704 triangles).
 bool coupling32_wanted(const stdg_ctx* c) { return !face_tiled_shape(c); }
-static bool face_shots_shape(const stdg_ctx* c) { return c->dim == 2 && c->Nphi == 6 && c->Ng == 3; }
-static bool coupling32_full(const stdg_ctx* c, int nshots) { return c->d_Kf32 && !(face_shots_shape(c) && nshots >= 16); }
-static bool coupling32_offdiag(const stdg_ctx* c, int nshots) { return c->d_Kf32 && !(face_shots_shape(c) && nshots >= 28); }
 
 cudaError_t launch_apply32(stdg_ctx* c, double dt, const float* x, float* y, double cfac, const int* xidx, int64_t ld,
                            int nshots) {
     const double scale = cfac * schur_c(c) * dt * dt;
-    if (coupling32_full(c, nshots)) return launch_coupling32(c, x, xidx, ld, nullptr, nullptr, 0, y, scale, nshots);
+    if (c->d_Kf32) return launch_coupling32(c, x, xidx, ld, nullptr, nullptr, 0, y, scale, nshots);
     STDG_DISPATCH(c->dim, c->Nphi, return (apply_tmpl<D_, N_, float>(c, c->d_D32, c->d_lamf32, c->d_muf32, c->d_rhoJ32, x, y, scale, true, true, xidx, ld, nshots)));
     return cudaSuccess;
 }
@@ -761,7 +755,7 @@ cudaError_t launch_apply_pre1(stdg_ctx* c, double dt, const double* y, const dou
 
 cudaError_t launch_apply_pre1_32(stdg_ctx* c, double dt, const float* y, const float* base, const int* bidx, int64_t bld,
                                  float* w, int nshots) {
-    if (!coupling32_offdiag(c, nshots)) return launch_apply32(c, dt, y, w, 1.0, nullptr, 0, nshots);
+    if (!c->d_Kf32) return launch_apply32(c, dt, y, w, 1.0, nullptr, 0, nshots);
     return launch_coupling32(c, y, nullptr, 0, base, bidx, bld, w, schur_c(c) * dt * dt, nshots);
 }
 

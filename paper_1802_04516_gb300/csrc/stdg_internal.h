@@ -253,6 +253,11 @@ bool launch_face_fast(stdg_ctx* c, const R* D, const R* lamf, const R* muf, cons
 cudaError_t launch_coupling_setup(stdg_ctx* c);
 cudaError_t launch_coupling_cast(stdg_ctx* c);
 cudaError_t launch_cast32(stdg_ctx* c, const double* a, float* b, int64_t n);   // kernels.cu
+// coupling_shots.cu: stacked shots at 2D p = p_gamma = 2, one lane per shot
+bool coupling_shots_applies(const stdg_ctx* c, int nshots, const float* x, int64_t ld, const float* base, int64_t bld,
+                            const float* y);
+cudaError_t launch_coupling_shots(stdg_ctx* c, const float* x, const int* xidx, int64_t ld, const float* base, const int* bidx,
+                                  int64_t bld, float* y, double scale, int nshots);
 bool coupling32_wanted(const stdg_ctx* c);   // whether this shape's FP32 operator uses them (kernels.cu)
 cudaError_t launch_coupling(stdg_ctx* c, const double* x, const int* xidx, int64_t ld, const double* base, const int* bidx,
                             int64_t bld, double* y, double scale, int nshots);
