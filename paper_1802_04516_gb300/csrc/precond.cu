@@ -225,67 +225,9 @@ __global__ void pre1_time_kernel(int64_t nq, int NG, const RefTables* __restrict
         for (int b = 0; b < NG; ++b) B[i * NG * NG + a * NG + b] = (R)A[a][NG + b];
 }
 
-// z_e = V (blockdiag B) V^T r_e for every element; r, z layout [e][k][a][n].  One warp per
-// element; V staged in shared memory with a padded row stride.
-template <typename R>
-__global__ void __launch_bounds__(128) pre1_apply_kernel(int64_t n_elem, int dim, int NP, int NG, const R* __restrict__ V,
-                                                         const R* __restrict__ B, const R* __restrict__ r0,
-                                                         const int* __restrict__ ridx, int64_t ld_vec, R* __restrict__ z0,
-                                                         int nshots, int64_t nvec) {
-    const R* r = r0;
-    extern __shared__ unsigned char smraw[];
-    R* sm = reinterpret_cast<R*>(smraw);
-    if (ridx) r += (int64_t)(*ridx) * ld_vec;
-    const int n = dim * NP;
-    const int ldv = n + 1;
-    const int per = n * ldv + 2 * n * NG;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    R* sV = sm + warp * per;
-    R* sr = sV + n * ldv;        // [(k,n)][a]
-    R* sw = sr + n * NG;         // [q][a]
-    for (int64_t e = blockIdx.x * (int64_t)wpb + warp; e < n_elem; e += (int64_t)gridDim.x * wpb) {
-        const R* Vg = V + e * (int64_t)n * n;
-        for (int t = lane; t < n * n; t += 32) sV[(t / n) * ldv + t % n] = Vg[t];
-        for (int shot = 0; shot < nshots; ++shot) {
-        const R* re = r + (int64_t)shot * nvec + e * (int64_t)n * NG;
-        R* z = z0 + (int64_t)shot * nvec;
-        for (int t = lane; t < n * NG; t += 32) {
-            const int k = t / (NG * NP), a = (t / NP) % NG, nn = t % NP;
-            sr[(k * NP + nn) * NG + a] = re[t];
-        }
-        __syncwarp();
-        for (int q = lane; q < n; q += 32) {
-            R u[kMaxNG];
-            for (int a = 0; a < NG; ++a) u[a] = 0;
-            for (int row = 0; row < n; ++row) {
-                const R v = sV[row * ldv + q];
-                for (int a = 0; a < NG; ++a) u[a] += v * sr[row * NG + a];
-            }
-            const R* Bq = B + (e * n + q) * NG * NG;
-            for (int a = 0; a < NG; ++a) {
-                R s = 0;
-                for (int b = 0; b < NG; ++b) s += Bq[a * NG + b] * u[b];
-                sw[q * NG + a] = s;
-            }
-        }
-        __syncwarp();
-        R* ze = z + e * (int64_t)n * NG;
-        for (int row = lane; row < n; row += 32) {
-            R acc[kMaxNG];
-            for (int a = 0; a < NG; ++a) acc[a] = 0;
-            for (int q = 0; q < n; ++q) {
-                const R v = sV[row * ldv + q];
-                for (int a = 0; a < NG; ++a) acc[a] += v * sw[q * NG + a];
-            }
-            const int k = row / NP, nn = row % NP;
-            for (int a = 0; a < NG; ++a) ze[(k * NG + a) * NP + nn] = acc[a];
-        }
-        __syncwarp();
-        }   // shots
-    }
-}
-
-// Register-blocked variant for d*N_phi <= 32: lane q holds column q of V (for u = V^T r),
+// Register-blocked kernel, kept for several shots in 3D at p = p_gamma = 2 (d N_phi = 30 fills a warp;
+// four shots on 3,072 tetrahedra: 12.6 us against 14.7 with one thread per row, FP64 149 against 153 us):
+// lane q holds column q of V (for u = V^T r),
 // lane `row` holds row `row` of V (for z = V w); the rows of r and w are read from shared
 // memory by all lanes at once (broadcast), so the inner loops are FMAs.
 template <int DIM, int NP, int NG, typename R>
@@ -722,18 +664,12 @@ static bool pre1_apply_fast(stdg_ctx* c, const R* V, const R* B, const R* r, R* 
             return true;
         }
     }
-#define STDG_PRE_FAST(D_, NP_, NG_)                                                                        \
-    if (d == D_ && np == NP_ && ng == NG_) {                                                              \
-        pre1_apply_reg_kernel<D_, NP_, NG_, R><<<(unsigned)blocks, 128, 0, c->stream>>>(c->n_elem, V, B, r, ridx, ld, z, nshots, c->nvel); \
-        note_launch(c);                                                                                    \
-        *err = cudaGetLastError();                                                                         \
-        return true;                                                                                       \
+    if (d == 3 && np == 10 && ng == 3 && nshots > 1) {
+        pre1_apply_reg_kernel<3, 10, 3, R><<<(unsigned)blocks, 128, 0, c->stream>>>(c->n_elem, V, B, r, ridx, ld, z, nshots, c->nvel);
+        note_launch(c);
+        *err = cudaGetLastError();
+        return true;
     }
-    STDG_PRE_FAST(2, 10, 4)
-    STDG_PRE_FAST(2, 6, 3)
-    STDG_PRE_FAST(3, 10, 3)
-    STDG_PRE_FAST(2, 3, 1)
-#undef STDG_PRE_FAST
     return false;
 }
 
@@ -772,14 +708,8 @@ static cudaError_t pre1_apply_t(stdg_ctx* c, const R* V, const R* B, const R* r,
                                 int nshots) {
     cudaError_t fe;
     if (pre1_apply_fast<R>(c, V, B, r, z, ridx, ld, &fe, nshots)) return fe;
-    const int n = c->dim * c->Nphi;
-    const int wpb = 4;
-    const size_t smem = sizeof(R) * (size_t)wpb * (n * (n + 1) + 2 * n * c->Ng);
-    cudaFuncSetAttribute(pre1_apply_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int64_t blocks = std::min<int64_t>((c->n_elem + wpb - 1) / wpb, 1 << 30);
-    pre1_apply_kernel<R><<<(unsigned)blocks, 32 * wpb, smem, c->stream>>>(c->n_elem, c->dim, c->Nphi, c->Ng, V, B, r, ridx, ld, z,
-                                                                          nshots, c->nvel); note_launch(c);
-    return cudaGetLastError();
+    if constexpr (std::is_same<R, float>::value) return launch_pre1_rows32(c, r, z, ridx, ld, nshots);
+    else return launch_pre1_rows(c, r, z, ridx, ld, nshots);
 }
 
 cudaError_t launch_pre1_apply(stdg_ctx* c, const double* r, double* z, const int* ridx, int64_t ld, int nshots) {

@@ -197,58 +197,49 @@ __global__ void __launch_bounds__(kP2Threads) pre2_setup_kernel(
     }
 }
 
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ double to_f(double v) { return v; }
-
-// z_e = S_e^{-1} (2 r_e - w_e), w = A P_1 r: one warp per element; lane holds rows lane + 32 i,
-// columns of S^{-1} (contiguous, blocks `es` entries apart) are streamed once per group of
-// SG shots.  R: arithmetic type, S: storage type of S^{-1}.
-template <typename R, typename S, int SG>
-__global__ void __launch_bounds__(128) pre2_local_kernel(int64_t n_elem, int N, int64_t es, const S* __restrict__ Sinv,
+// z_e = S_e^{-1} (2 r_e - w_e), w = A P_1 r, one thread per (element, row): consecutive threads are
+// consecutive rows of consecutive elements, so that whole warps work (a warp per element left 28 of 64
+// lanes idle at N = 36, and FP64 pays for idle lanes: 360 -> 99 us on 40,000 triangles at p = 2,
+// 124 -> 17 us at p = 1; FP32, 6 shots, p = 3 on 3,600 triangles: 139 -> 33 us).  The
+// columns of S^{-1} (contiguous, blocks `es` entries apart) are read once for SC shots; a single shot's
+// FP32 blocks normally come from their FP16 copy below.
+template <typename R, int SC>
+__global__ void __launch_bounds__(256) pre2_local_kernel(int64_t n_elem, int EB, int N, int64_t es, const R* __restrict__ Sinv,
                                                          const R* __restrict__ r, const int* __restrict__ ridx,
                                                          int64_t ld, const R* __restrict__ w, R* __restrict__ z,
                                                          int nshots, int64_t nvec) {
-    extern __shared__ unsigned char smraw[];
+    extern __shared__ __align__(16) unsigned char smraw[];
+    R* st = reinterpret_cast<R*>(smraw);          // [shot of the chunk][element][row]
     if (ridx) r += (int64_t)(*ridx) * ld;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    R* st = reinterpret_cast<R*>(smraw) + (size_t)warp * SG * N;
-    for (int64_t e = blockIdx.x * (int64_t)wpb + warp; e < n_elem; e += (int64_t)gridDim.x * wpb) {
-        const S* Se = Sinv + e * es;
-        for (int s0 = 0; s0 < nshots; s0 += SG) {
-            const int sg = min(SG, nshots - s0);
-            for (int q = lane; q < SG * N; q += 32) {
-                const int g = q / N, c = q % N;
-                const int64_t i = (int64_t)(s0 + g) * nvec + e * N + c;
-                st[q] = g < sg ? (R)2 * r[i] - w[i] : (R)0;
+    const int64_t e0 = (int64_t)blockIdx.x * EB;
+    const int ne = (int)min((int64_t)EB, n_elem - e0);
+    const int le = threadIdx.x / N, row = threadIdx.x - le * N;
+    const bool act = le < ne;
+    const R* Se = Sinv + (e0 + (act ? le : 0)) * es + row;
+    for (int s0 = 0; s0 < nshots; s0 += SC) {
+        if (s0) __syncthreads();
+        if (act) {
+#pragma unroll
+            for (int c = 0; c < SC; ++c) {
+                const int64_t i = (int64_t)(s0 + c) * nvec + (e0 + le) * N + row;
+                st[(c * EB + le) * N + row] = SC == 1 || s0 + c < nshots ? (R)2 * r[i] - w[i] : (R)0;
             }
-            __syncwarp();
-            R acc[kP2MaxRows][SG];
-#pragma unroll
-            for (int i = 0; i < kP2MaxRows; ++i)
-#pragma unroll
-                for (int g = 0; g < SG; ++g) acc[i][g] = 0;
-            for (int c = 0; c < N; ++c) {
-                const S* col = Se + (int64_t)c * N;
-#pragma unroll
-                for (int i = 0; i < kP2MaxRows; ++i) {
-                    const int rr = lane + 32 * i;
-                    if (rr < N) {
-                        const R a = (R)to_f(col[rr]);
-#pragma unroll
-                        for (int g = 0; g < SG; ++g) acc[i][g] = fma(a, st[g * N + c], acc[i][g]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < kP2MaxRows; ++i) {
-                const int rr = lane + 32 * i;
-                if (rr < N)
-#pragma unroll
-                    for (int g = 0; g < SG; ++g)
-                        if (g < sg) z[(int64_t)(s0 + g) * nvec + e * N + rr] = acc[i][g];
-            }
-            __syncwarp();
         }
+        __syncthreads();
+        if (!act) continue;
+        R acc[SC];
+#pragma unroll
+        for (int c = 0; c < SC; ++c) acc[c] = (R)0;
+        const R* sp = st + le * N;
+#pragma unroll 8
+        for (int q = 0; q < N; ++q) {
+            const R a = __ldg(Se + (int64_t)q * N);
+#pragma unroll
+            for (int c = 0; c < SC; ++c) acc[c] = fma(a, sp[c * EB * N + q], acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < SC; ++c)
+            if (SC == 1 || s0 + c < nshots) z[(int64_t)(s0 + c) * nvec + (e0 + le) * N + row] = acc[c];
     }
 }
 
@@ -387,17 +378,17 @@ cudaError_t launch_pre2_setup(stdg_ctx* c, double dt, int* d_status) {
     return cudaGetLastError();
 }
 
-template <typename R, typename S>
-static cudaError_t pre2_local_t(stdg_ctx* c, const S* Sinv, int64_t es, const R* r, const int* ridx, int64_t ld,
+template <typename R>
+static cudaError_t pre2_local_t(stdg_ctx* c, const R* Sinv, int64_t es, const R* r, const int* ridx, int64_t ld,
                                 const R* w, R* z, int nshots) {
     const int N = c->dim * c->Nphi * c->Ng;
     if constexpr (std::is_same<R, float>::value) {   // a batch of shots: one GEMM per element pair on the tensor cores
         cudaError_t e;
         if (nshots > 1 && launch_pre2_local_mma(c, r, ridx, ld, w, z, nshots, &e)) return e;
     }
-    const int wpb = c->tune.pre2_wpb;
-    const int64_t blocks = std::min<int64_t>((c->n_elem + wpb - 1) / wpb, 1 << 30);
-    if constexpr (std::is_same<R, float>::value && std::is_same<S, float>::value) {
+    if constexpr (std::is_same<R, float>::value) {
+        const int wpb = c->tune.pre2_wpb;
+        const int64_t blocks = std::min<int64_t>((c->n_elem + wpb - 1) / wpb, 1 << 30);
         // one shot with the FP16 copy of the blocks (half the bytes of the dominant stream)
         if (nshots == 1 && c->d_pre2_16 && c->pre2_bits == 16 && Sinv == c->d_pre2_32) {
             pre2_local_half_kernel<<<(unsigned)blocks, 32 * wpb, sizeof(float) * wpb * N, c->stream>>>(
@@ -406,13 +397,22 @@ static cudaError_t pre2_local_t(stdg_ctx* c, const S* Sinv, int64_t es, const R*
             return cudaGetLastError();
         }
     }
-    if (nshots == 1) {
-        pre2_local_kernel<R, S, 1><<<(unsigned)blocks, 32 * wpb, sizeof(R) * wpb * N, c->stream>>>(
-            c->n_elem, N, es, Sinv, r, ridx, ld, w, z, nshots, c->nvel);
-    } else {
-        pre2_local_kernel<R, S, 4><<<(unsigned)blocks, 32 * wpb, sizeof(R) * wpb * 4 * N, c->stream>>>(
-            c->n_elem, N, es, Sinv, r, ridx, ld, w, z, nshots, c->nvel);
+    // whole warps of rows, at most 256 threads, at least one block per SM on small meshes
+    const int most = (int)std::max<int64_t>(1, std::min<int64_t>(256 / N, c->n_elem / c->n_sm));
+    double best = 0.0;
+    int EB = 1;
+    for (int e2 = 1; e2 <= most; ++e2) {
+        const double eff = (double)(e2 * N) / ((e2 * N + 31) / 32 * 32);
+        if (eff >= best) { best = eff; EB = e2; }
     }
+    const unsigned grid = (unsigned)((c->n_elem + EB - 1) / EB);
+    const int threads = (EB * N + 31) / 32 * 32;
+    auto go = [&](auto kern, int SC) {
+        kern<<<grid, threads, sizeof(R) * SC * EB * N, c->stream>>>(c->n_elem, EB, N, es, Sinv, r, ridx, ld, w, z, nshots, c->nvel);
+    };
+    if (nshots == 1) go(pre2_local_kernel<R, 1>, 1);
+    else if (nshots <= 4) go(pre2_local_kernel<R, 4>, 4);
+    else go(pre2_local_kernel<R, 8>, 8);
     note_launch(c);
     return cudaGetLastError();
 }
@@ -421,21 +421,21 @@ static cudaError_t pre2_local_t(stdg_ctx* c, const S* Sinv, int64_t es, const R*
 cudaError_t launch_pre2_local(stdg_ctx* c, int fp32, const void* r, const void* w, void* z) {
     const int64_t N = c->dim * c->Nphi * c->Ng;
     if (fp32)
-        return pre2_local_t<float, float>(c, c->d_pre2_32, pre2_stride32(c), (const float*)r, nullptr, 0,
+        return pre2_local_t<float>(c, c->d_pre2_32, pre2_stride32(c), (const float*)r, nullptr, 0,
                                            (const float*)w, (float*)z, 1);
-    return pre2_local_t<double, double>(c, c->d_pre2, N * N, (const double*)r, nullptr, 0, (const double*)w, (double*)z, 1);
+    return pre2_local_t<double>(c, c->d_pre2, N * N, (const double*)r, nullptr, 0, (const double*)w, (double*)z, 1);
 }
 
 // the element-local step alone for all the context's shots, FP32 (the tensor-core kernel
 // for a batch of shots where it applies)
 cudaError_t launch_pre2_local_batch(stdg_ctx* c, const float* r, const float* w, float* z) {
-    return pre2_local_t<float, float>(c, c->d_pre2_32, pre2_stride32(c), r, nullptr, 0, w, z, c->n_shots);
+    return pre2_local_t<float>(c, c->d_pre2_32, pre2_stride32(c), r, nullptr, 0, w, z, c->n_shots);
 }
 
 // z = P_2 r for nshots stacked shots: y = P_1 r, w = A y, z = S^{-1} (2 r - w).
 // Since D_i y_i = r_i, A y = r + sum_e N_{i,e} y_e: only the neighbour couplings are applied.
-template <typename R, typename S>
-static cudaError_t pre2_apply_t(stdg_ctx* c, const S* Sinv, int64_t es, const R* r, R* z, const int* ridx, int64_t ld,
+template <typename R>
+static cudaError_t pre2_apply_t(stdg_ctx* c, const R* Sinv, int64_t es, const R* r, R* z, const int* ridx, int64_t ld,
                                 int nshots, bool fp32) {
     R* y = reinterpret_cast<R*>(c->d_p2y);
     R* w = reinterpret_cast<R*>(c->d_p2t);
@@ -449,16 +449,16 @@ static cudaError_t pre2_apply_t(stdg_ctx* c, const S* Sinv, int64_t es, const R*
         if ((e = launch_apply_pre1(c, c->pre_dt, (const double*)y, (const double*)r, ridx, ld, (double*)w, nshots)) != cudaSuccess)
             return e;
     }
-    return pre2_local_t<R, S>(c, Sinv, es, r, ridx, ld, w, z, nshots);
+    return pre2_local_t<R>(c, Sinv, es, r, ridx, ld, w, z, nshots);
 }
 
 cudaError_t launch_pre2_apply(stdg_ctx* c, const double* r, double* z, const int* ridx, int64_t ld, int nshots) {
     const int64_t N = c->dim * c->Nphi * c->Ng;
-    return pre2_apply_t<double, double>(c, c->d_pre2, N * N, r, z, ridx, ld, nshots, false);
+    return pre2_apply_t<double>(c, c->d_pre2, N * N, r, z, ridx, ld, nshots, false);
 }
 
 cudaError_t launch_pre2_apply32(stdg_ctx* c, const float* r, float* z, const int* ridx, int64_t ld, int nshots) {
-    return pre2_apply_t<float, float>(c, c->d_pre2_32, pre2_stride32(c), r, z, ridx, ld, nshots, true);
+    return pre2_apply_t<float>(c, c->d_pre2_32, pre2_stride32(c), r, z, ridx, ld, nshots, true);
 }
 
 }  // namespace stdg

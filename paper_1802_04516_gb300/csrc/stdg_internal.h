@@ -267,6 +267,8 @@ cudaError_t launch_coupling32(stdg_ctx* c, const float* x, const int* xidx, int6
 // precond.cu
 cudaError_t launch_pre1_setup(stdg_ctx* c, const double* d_Rinv, const int32_t* d_elem_face, int* d_status);
 cudaError_t launch_pre1_time(stdg_ctx* c, double dt);
+cudaError_t launch_pre1_rows(stdg_ctx* c, const double* r, double* z, const int* ridx, int64_t ld, int nshots);
+cudaError_t launch_pre1_rows32(stdg_ctx* c, const float* r, float* z, const int* ridx, int64_t ld, int nshots);
 cudaError_t launch_pre1_apply(stdg_ctx* c, const double* r, double* z, const int* ridx, int64_t ld, int nshots = 1);
 cudaError_t launch_pre1_apply32(stdg_ctx* c, const float* r, float* z, const int* ridx, int64_t ld, int nshots = 1);
 
