@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <type_traits>
 
 #include "stdg_internal.h"
 
@@ -419,65 +420,123 @@ cudaError_t launch_to_fp32(stdg_ctx* c) {
 // ---------------------------------------------------------------------------------
 // y[e][k][a][n] = rho_i |J_i| sum_b T[a][b] sum_n' Mref[n][n'] v[e][k][b][n']
 // n_elem = elements x shots of the (shot-major) vectors, n_elem_base = elements of the mesh.
-// A block takes EB = blockDim / (d N_gamma) consecutive elements at a time: their values are
-// loaded into shared memory with consecutive (coalesced) reads, each thread forms one row
-// (k, a) of one element, the rows go back to the same shared buffer and out with consecutive
-// writes.
-template <int NP, typename R>
-__global__ void __launch_bounds__(128) mass_kernel(int64_t n_elem, int64_t n_elem_base, int dim, int NG,
-                                                   const RefTables* __restrict__ rtp, const R* __restrict__ rhoJ,
-                                                   const R* __restrict__ v, const int* __restrict__ vidx, int64_t ld,
-                                                   R* __restrict__ y) {
+//
+// FP32 kernel of the shapes whose face term runs in a tiled face kernel (N_phi = 10).  A thread takes
+// one row (e, k): its N_gamma x N_phi values in registers, M_ref and T as kernel arguments, so that a
+// product reads its second operand from the constant bank and shared memory only transposes.  A warp
+// takes 32 consecutive rows, copied by cp.async in order into rows of an odd number of pieces (no bank
+// conflicts), one group ahead; the results leave through the same buffer with consecutive stores.
+// Bound by HBM at size.  200,704 triangles, p = p_gamma = 3: MASSNEW us against 70 us for a block per 16
+// elements with one thread per (k, a) row reading M_ref and the values from shared memory; 82,944
+// tetrahedra, p = p_gamma = 2: MASSNEW3 against 35 us.  Same sums in the same order.
+template <int NP, int NG>
+struct MassTables { float M[NP * NP], T[NG * NG]; };
+
+template <int NP, int NG>
+struct MassWarp {
+    static constexpr int NV = NP * NG;                               // values per row (e, k)
+    static constexpr int PW = NV % 4 == 0 ? 4 : 2;                   // floats per piece (16 or 8 bytes)
+    static constexpr int PR = NV / PW;                               // pieces per row
+    static constexpr int PITCH = (PR % 2 ? PR : PR + 1) * PW;        // floats per staged row
+    static constexpr int BUF = 32 * PITCH;
+};
+
+template <int NP, int NG>
+__global__ void __launch_bounds__(128) mass_warp_kernel(int64_t n_rows, int dim, int64_t n_elem_base,
+                                                        const __grid_constant__ MassTables<NP, NG> tab,
+                                                        const float* __restrict__ rhoJ, const float* __restrict__ v,
+                                                        const int* __restrict__ vidx, int64_t ld, float* __restrict__ y) {
+    using L = MassWarp<NP, NG>;
+    constexpr int NV = L::NV, PW = L::PW, PR = L::PR, PITCH = L::PITCH;
+    __shared__ __align__(16) float stage[4][2][L::BUF];
     if (vidx) v += (int64_t)(*vidx) * ld;
-    extern __shared__ __align__(16) unsigned char mass_smem[];
-    R* sV = reinterpret_cast<R*>(mass_smem);
-    __shared__ R sM[NP * NP];
-    __shared__ R sT[kMaxNG * kMaxNG];
-    for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sM[t] = (R)rtp->Mref[t];
-    for (int t = threadIdx.x; t < NG * NG; t += blockDim.x) sT[t] = (R)rtp->T[t];
-    const int rows_e = dim * NG, per_e = rows_e * NP;
-    const int EB = blockDim.x / rows_e;
-    const int r = threadIdx.x, le = r / rows_e, ka = r % rows_e, k = ka / NG, a = ka % NG;
-    for (int64_t e0 = blockIdx.x * (int64_t)EB; e0 < n_elem; e0 += (int64_t)gridDim.x * EB) {
-        const int ne = (int)min((int64_t)EB, n_elem - e0);
-        const int64_t base = e0 * per_e;
-        __syncthreads();   // the previous elements' values have been written out
-        for (int t = threadIdx.x; t < ne * per_e; t += blockDim.x) sV[t] = v[base + t];
-        __syncthreads();
-        const bool act = le < ne;
-        R out[NP];
-        if (act) {
-            const R* ve = sV + (le * dim + k) * NG * NP;
-            R tv[NP];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t n_grp = (n_rows + 31) / 32, W = (int64_t)gridDim.x * 4;
+    auto issue = [&](int64_t g, int b) {
+        if (g < n_grp) {
+            const int64_t p0 = g * 32 * PR, pn = n_rows * PR;
 #pragma unroll
-            for (int n = 0; n < NP; ++n) tv[n] = 0;
-            for (int b = 0; b < NG; ++b) {
-                const R tab = sT[a * NG + b];
-#pragma unroll
-                for (int n = 0; n < NP; ++n) tv[n] += tab * ve[b * NP + n];
+            for (int u = 0; u < PR; ++u) {
+                const int p = u * 32 + lane, r = p / PR, j = p % PR;
+                const bool ok = p0 + p < pn;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(&stage[warp][b][r * PITCH + j * PW])),
+                             "l"(v + (ok ? (p0 + p) * PW : 0)), "n"(4 * PW), "r"(ok ? 4 * PW : 0)
+                             : "memory");
             }
-            const R sc = rhoJ[(e0 + le) % n_elem_base];
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int64_t g = blockIdx.x * 4LL + warp;
+    issue(g, 0);
+    for (int b = 0; g < n_grp; g += W, b ^= 1) {
+        issue(g + W, b ^ 1);
+        const int64_t row = g * 32 + lane;
+        const float sc = row < n_rows ? rhoJ[row / dim % n_elem_base] : 0.f;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        float* mine = &stage[warp][b][lane * PITCH];
+        float x[NV];
+#pragma unroll
+        for (int j = 0; j < PR; ++j) {
+            if constexpr (PW == 4) {
+                const float4 q = reinterpret_cast<const float4*>(mine)[j];
+                x[4 * j] = q.x; x[4 * j + 1] = q.y; x[4 * j + 2] = q.z; x[4 * j + 3] = q.w;
+            } else {
+                const float2 q = reinterpret_cast<const float2*>(mine)[j];
+                x[2 * j] = q.x; x[2 * j + 1] = q.y;
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < NG; ++a) {
+            float tv[NP];
 #pragma unroll
             for (int n = 0; n < NP; ++n) {
-                R acc = 0;
+                tv[n] = 0.f;
 #pragma unroll
-                for (int q = 0; q < NP; ++q) acc += sM[n * NP + q] * tv[q];
-                out[n] = sc * acc;
+                for (int q = 0; q < NG; ++q) tv[n] += tab.T[a * NG + q] * x[q * NP + n];
+            }
+#pragma unroll
+            for (int n = 0; n < NP; n += 2) {
+                float o[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float acc = 0.f;
+#pragma unroll
+                    for (int q = 0; q < NP; ++q) acc += tab.M[(n + u) * NP + q] * tv[q];
+                    o[u] = sc * acc;
+                }
+                *reinterpret_cast<float2*>(mine + a * NP + n) = make_float2(o[0], o[1]);
             }
         }
-        __syncthreads();   // every row has read the element's values
-        if (act) {
+        __syncwarp();
+        const int64_t p0 = g * 32 * PR, pn = n_rows * PR;
 #pragma unroll
-            for (int n = 0; n < NP; ++n) sV[r * NP + n] = out[n];   // row (e, k, a) of y
+        for (int u = 0; u < PR; ++u) {
+            const int p = u * 32 + lane, r = p / PR, j = p % PR;
+            if (p0 + p < pn) {
+                const float* src = &stage[warp][b][r * PITCH + j * PW];
+                if constexpr (PW == 4) *reinterpret_cast<float4*>(y + (p0 + p) * 4) = *reinterpret_cast<const float4*>(src);
+                else *reinterpret_cast<float2*>(y + (p0 + p) * 2) = *reinterpret_cast<const float2*>(src);
+            }
         }
-        __syncthreads();
-        for (int t = threadIdx.x; t < ne * per_e; t += blockDim.x) y[base + t] = sV[t];
+        __syncwarp();   // the buffer is free for the group after next
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// Row-per-thread variant for stacked shots: thread (element, k, a) reads the element's rows
-// directly; with many shots the grid streams long contiguous vectors and this form measured
-// faster than the staged one (1.17 -> 0.91 ms per launch for 64 shots on 200,704 triangles).
+template <int NP, int NG>
+static void mass_warp(stdg_ctx* c, const float* rhoJ, const float* x, const int* xidx, int64_t ld, float* y, int nshots) {
+    MassTables<NP, NG> t;
+    for (int i = 0; i < NP * NP; ++i) t.M[i] = (float)c->rt.Mref[i];
+    for (int i = 0; i < NG * NG; ++i) t.T[i] = (float)c->rt.T[i];
+    const int64_t rows = c->n_elem * nshots * c->dim;
+    mass_warp_kernel<NP, NG><<<(unsigned)std::min<int64_t>((rows + 127) / 128, (int64_t)c->n_sm * 8), 128, 0, c->stream>>>(
+        rows, c->dim, c->n_elem, t, rhoJ, x, xidx, ld, y);
+    note_launch(c);
+}
+
+// Any shape: thread (element, k, a) reads the element's rows directly.
 template <int NP, typename R>
 __global__ void mass_rows_kernel(int64_t n_elem, int64_t n_elem_base, int dim, int NG, const RefTables* __restrict__ rtp,
                                  const R* __restrict__ rhoJ, const R* __restrict__ v, const int* __restrict__ vidx,
@@ -677,14 +736,18 @@ static cudaError_t apply_tmpl(stdg_ctx* c, const R* D, const R* lamf, const R* m
     if (mass) {
         const int64_t rows = c->n_elem * nshots * c->dim * NG;
         const int64_t ne = c->n_elem * nshots;
-        if (nshots > 1) {
+        bool done = false;
+        if constexpr (std::is_same<R, float>::value && NP == 10) {
+            const bool al = reinterpret_cast<uintptr_t>(x) % 16 == 0 && reinterpret_cast<uintptr_t>(y) % 16 == 0 && ld % 4 == 0;
+            if (al && face_tiled_shape(c)) {
+                if (DIM == 2) mass_warp<10, 4>(c, rhoJ, x, xidx, ld, y, nshots);
+                else mass_warp<10, 3>(c, rhoJ, x, xidx, ld, y, nshots);
+                done = true;
+            }
+        }
+        if (!done) {
             mass_rows_kernel<NP, R><<<(unsigned)std::min<int64_t>((rows + 127) / 128, c->n_sm * 64), 128, 0, c->stream>>>(
                 ne, c->n_elem, c->dim, NG, c->d_rt, rhoJ, x, xidx, ld, y); note_launch(c);
-        } else {
-            const int EB = 128 / (c->dim * NG);   // elements per block and pass (d N_gamma <= 15)
-            const size_t smem = sizeof(R) * (size_t)EB * c->dim * NG * NP;
-            mass_kernel<NP, R><<<(unsigned)std::min<int64_t>((ne + EB - 1) / EB, (int64_t)c->n_sm * 16), 128, smem,
-                                 c->stream>>>(ne, c->n_elem, c->dim, NG, c->d_rt, rhoJ, x, xidx, ld, y); note_launch(c);
         }
     }
     if (!face) return cudaGetLastError();
