@@ -800,7 +800,14 @@ cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, dou
 // faster (264 against 325 us on 200,704 triangles) but move the mixed slab of the sliver mesh by more
 // than two runs differ (its inner residual is met by a different iterate; single velocities by 3e-7).
 // Elsewhere they win at every size (2D p = 2: 117 against 238 us on 200,704 triangles).
-bool coupling32_wanted(const stdg_ctx* c) { return !face_tiled_shape(c); }
+// In 3D with one time node D~ is read for few products and the couplings only win while they stay in
+// L2 (CG iteration at p = 2: 60 against 61 us on 4,374 tetrahedra = 79 MB, 120 against 92 us on 10,368; p = 1:
+// 42 against 56 us at 30 MB, 153 against 140 us at 138 MB).
+bool coupling32_wanted(const stdg_ctx* c) {
+    if (face_tiled_shape(c)) return false;
+    const int64_t n2 = (int64_t)c->dim * c->Nphi * c->dim * c->Nphi;
+    return !(c->dim == 3 && c->Ng == 1 && (int64_t)sizeof(float) * n2 * (2 * c->n_face + c->n_elem) > (80LL << 20));
+}
 
 cudaError_t launch_apply32(stdg_ctx* c, double dt, const float* x, float* y, double cfac, const int* xidx, int64_t ld,
                            int nshots) {

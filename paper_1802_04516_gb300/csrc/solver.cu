@@ -27,49 +27,10 @@
 #include <cmath>
 #include <cstring>
 
+#include "krylov.h"
 #include "stdg_internal.h"
 
 namespace stdg {
-
-constexpr int kMaxRestart = 64;
-constexpr int kRedThreads = 256;
-constexpr int kFinThreads = 1024;   // single-block reduction / control kernels
-constexpr int kDotChunk = 16;       // basis vectors per pass of the multi-dot kernels
-constexpr int kDotLoads = 8;        // basis vectors whose values a thread has in flight at once
-
-// Krylov state of one shot
-struct ShotScalars {
-    double bnorm, tol_abs;
-    double rr, pq, alpha, beta;                   // CG
-    double gbeta, resid;                          // GMRES
-    double hcol[kMaxRestart + 2], hpass[kMaxRestart + 2];
-    double H[(kMaxRestart + 1) * kMaxRestart];
-    double cs[kMaxRestart], sn[kMaxRestart], g[kMaxRestart + 1], y[kMaxRestart];
-    double red[3];                                // reduced sums handed between warps
-    double vscale;                                // 1 / ||w||, the scale of the next basis vector
-    int jj;            // basis columns this shot uses in the current cycle
-    int active;        // still iterating in the current cycle / CG solve
-    int reorth;        // this Arnoldi step needs the second Gram-Schmidt pass
-    int converged, zero_x;                        // zero_x: b_s = 0, so x_s = 0
-    // FP64 refinement level (mixed precision)
-    double ir_bnorm, ir_tol_abs, ir_rnorm, ir_scale;
-    int ir_conv, ir_zero;
-};
-
-// Recorded bodies whose executions are counted on the device: the kernels launched by a call are
-// sum_i runs[i] * (kernels of body i), the second factor known from recording.
-enum Body { kBodyStraight, kBodyIr, kBodyCycle, kBodyInner, kBodies };
-
-// loop control shared by all shots
-struct DevScalars {
-    int j, iters, flag_outer, flag_inner, max_iters, m;
-    int any;           // a shot still iterates (collected by the shots' last blocks)
-    int ir_flag, ir_count, ir_max;
-    // statistics, reset by the host before a batch of steps
-    int st_total, st_max, st_refine, st_notconv, st_nonfinite;
-    double st_final_rel, st_iters_sum;
-    unsigned int runs[kBodies];       // executions of each recorded body since the last reset
-};
 
 struct Workspace {
     int m = 30;
@@ -84,6 +45,8 @@ struct Workspace {
     double* partials = nullptr;   // [slot][shot][block], (kMaxRestart + 2) slots
     unsigned* done = nullptr;     // [ns] blocks of a shot, [1] shots that have finished a reducing kernel
     double* dparams = nullptr;    // t^n, dt, step index
+    double *pb = nullptr;         // second search direction of the fused CG
+    float *pb32 = nullptr;
     double *V = nullptr, *w = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *t = nullptr;   // FP64
     float *V32 = nullptr, *w32 = nullptr, *b32 = nullptr, *x32 = nullptr, *r32 = nullptr, *p32 = nullptr, *q32 = nullptr;
     float *z32 = nullptr, *t32 = nullptr;
@@ -102,128 +65,6 @@ struct Workspace {
 };
 
 static Workspace* W(stdg_ctx* c) { return reinterpret_cast<Workspace*>(c->ws); }
-
-// ---------------------------------------------------------------------------------
-// reductions
-// ---------------------------------------------------------------------------------
-__device__ __forceinline__ double block_sum(double v) {
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    double s = 0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-    return s;   // valid in thread 0
-}
-
-// sum of p[0..n) by one warp; valid in every lane (read past L1: the values may come from other
-// blocks of the same kernel)
-__device__ __forceinline__ double warp_sum(const double* p, int n) {
-    double v = 0;
-    for (int i = threadIdx.x & 31; i < n; i += 32) v += __ldcg(p + i);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// partial sums of slot k, shot s: part + (k * ns + s) * G
-__device__ __forceinline__ const double* slot(const double* part, int k, int s, int ns, int G) {
-    return part + ((int64_t)k * ns + s) * G;
-}
-
-// Per-thread dot-product accumulator: FP64 for FP64 vectors; for FP32 vectors an error-free
-// (TwoProduct + TwoSum) pair of floats, so FP32 inner products carry FP64-level accuracy
-// without FP64 arithmetic (GB300's FP64 rate is 1/64 of FP32).
-template <typename R> struct Acc;
-template <> struct Acc<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-    __device__ __forceinline__ double value() const { return s; }
-    __device__ __forceinline__ void plus_xor(const Acc& give, int o) { s += __shfl_xor_sync(0xffffffffu, give.s, o); }
-};
-template <> struct Acc<float> {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float a, float b) {
-        const float p = a * b;
-        const float pe = fmaf(a, b, -p);
-        const float t = s + p;
-        const float z = t - s;
-        const float te = (s - (t - z)) + (p - z);
-        s = t;
-        c += te + pe;
-    }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-    // adds the pair `give` of lane ^ o (TwoSum of the leading terms): the tree over the lanes stays in
-    // float pairs, because at two FP64 lanes an SM the conversions and FP64 additions of 16 sums per
-    // thread took 5 us a block, more than the products
-    __device__ __forceinline__ void plus_xor(const Acc& give, int o) {
-        const float os = __shfl_xor_sync(0xffffffffu, give.s, o), oc = __shfl_xor_sync(0xffffffffu, give.c, o);
-        const float t = s + os;
-        const float z = t - s;
-        c += oc + ((s - (t - z)) + (os - z));
-        s = t;
-    }
-};
-
-// True in every thread of the block that arrives last of `total` (its reads then see what the
-// others wrote before arriving).  Reductions finish in that block, in a fixed order, instead of in
-// a single-block kernel of their own: a dependent launch costs 2-3 us and such a kernel took
-// 8-13 us, five of them per GMRES iteration.  The counter is back at zero afterwards.
-__device__ __forceinline__ bool last_block(unsigned* counter, unsigned total) {
-    __shared__ bool last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicInc(counter, total - 1) == total - 1;
-    __syncthreads();
-    if (last) __threadfence();
-    return last;
-}
-
-// Block-wide sums of the 16 accumulators that each thread holds: the lanes of a warp halve their
-// set at every exchange (16 exchanges instead of 80), then FP64 sums over the warps through shared
-// memory.  The sum of accumulator k is valid in thread k < 16.
-template <typename R>
-__device__ __forceinline__ double block_sum16(Acc<R> (&v)[kDotChunk]) {
-    __shared__ double red[32][kDotChunk];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16, n = kDotChunk / 2; o > 1; o >>= 1, n >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const Acc<R> give = up ? v[i] : v[i + n];
-            if (up) v[i] = v[i + n];
-            v[i].plus_xor(give, o);
-        }
-    }
-    v[0].plus_xor(v[0], 1);
-    const int k = (lane & 16 ? 8 : 0) + (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
-    __syncthreads();
-    if ((lane & 1) == 0) red[warp][k] = v[0].value();
-    __syncthreads();
-    double s = 0;
-    if (threadIdx.x < kDotChunk)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
-    return s;
-}
-
-// Block-wide sum of one accumulator; valid in thread 0.
-template <typename R>
-__device__ __forceinline__ double block_sum1(Acc<R> v) {
-    __shared__ double red[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v.plus_xor(v, o);
-    __syncthreads();
-    if (lane == 0) red[warp] = v.value();
-    __syncthreads();
-    double s = 0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    return s;
-}
 
 // 16-byte vector access: VW = 4 floats or 2 doubles per load/store.  Every pointer that is
 // vectorised is 16-byte aligned (separate allocations, or basis columns at a leading
@@ -278,10 +119,6 @@ template <typename R>
 __device__ __forceinline__ void put_acc(double* part, int k, const Acc<R>& v) {
     const double s = block_sum1(v);
     if (threadIdx.x == 0) part[((int64_t)k * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
-}
-
-__device__ __forceinline__ void set_cond(cudaGraphConditionalHandle h, int use, int v) {
-    if (use) cudaGraphSetConditional(h, v ? 1u : 0u);
 }
 
 // per-shot dot products a_s . b_s into slot k
@@ -1092,7 +929,7 @@ struct Flow {
 
 // ---- (P)CG on vectors of type R; apply(x, y): y = A x; prec(r, z): z = P^{-1} r or null --------
 template <typename R, class Apply, class Prec>
-static void solve_cg(Flow& F, Apply apply, Prec prec, bool use_prec, const R* b, R* x, R* r, R* p, R* q, R* z,
+static void solve_cg(Flow& F, double dt, Apply apply, Prec prec, bool use_prec, const R* b, R* x, R* r, R* p, R* pb, R* q, R* z,
                      double rel_tol, int max_iters, double bnorm_given, int gate_ir) {
     stdg_ctx* c = F.c;
     Workspace* ws = F.ws;
@@ -1100,6 +937,7 @@ static void solve_cg(Flow& F, Apply apply, Prec prec, bool use_prec, const R* b,
     const int ns = ws->ns, G = (int)ws->G;
     const dim3 grid = ws->grid();
     R* zz = use_prec ? z : r;
+    const bool fused = use_prec && cg_fused_applies(c, ns, sizeof(R) == 4);   // two kernels an iteration
     F.loop(kBodyInner, &ws->sc->flag_inner,
            [&](cudaGraphConditionalHandle h, int use) {
                F.check(apply(x, q));
@@ -1111,6 +949,10 @@ static void solve_cg(Flow& F, Apply apply, Prec prec, bool use_prec, const R* b,
                copy_kernel<R><<<ws->red_blocks, kRedThreads, 0, c->stream>>>(n, zz, p); note_launch(c);
            },
            [&](cudaGraphConditionalHandle h, int use) {
+               if (fused) {
+                   F.check(launch_cg_fused(c, dt, x, r, zz, p, pb, q, ws->sc, ws->ss, ws->partials, ws->done, h, use));
+                   return;
+               }
                F.check(apply(p, q));
                cg_dot_alpha_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, p, q, ws->partials, ws->ss, ws->done); note_launch(c);
                cg_update_kernel<R><<<grid, kRedThreads, 0, c->stream>>>(nv, ws->ss, x, r, p, q, ws->partials); note_launch(c);
@@ -1220,7 +1062,7 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
     const double tol = c->opt.rel_tol;
     const int maxit = c->opt.max_iters;
     if (c->opt.precision == STDG_FP64) {
-        if (cn) solve_cg<double>(F, A64, P64c, pre, b, x, ws->r, ws->p, ws->q, ws->z, tol, maxit, -1.0, 0);
+        if (cn) solve_cg<double>(F, dt, A64, P64c, pre, b, x, ws->r, ws->p, ws->pb, ws->q, ws->z, tol, maxit, -1.0, 0);
         else solve_gmres<double>(F, A64, A64i, AP64, P64, pre, b, x, ws->V, ws->w, ws->z, ws->t, tol, maxit, -1.0, 0);
         zero_if_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, x, ws->ss, 0); note_launch(c);
         solve_stats_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ns, cn ? 1 : 0); note_launch(c);
@@ -1239,7 +1081,7 @@ static void record_solve(Flow& F, double dt, double* b, double* x) {
                ir_check_kernel<<<1, ws->fin_threads(), 0, c->stream>>>(ws->sc, ws->ss, ws->partials, ns, G, maxit); note_launch(c);
                ir_convert_kernel<<<grid, kRedThreads, 0, c->stream>>>(nv, ws->sc, ws->ss, ws->r, ws->b32, ws->x32); note_launch(c);
                if (cn)
-                   solve_cg<float>(F, A32, P32c, pre, ws->b32, ws->x32, ws->r32, ws->p32, ws->q32, ws->z32, c->opt.inner_tol,
+                   solve_cg<float>(F, dt, A32, P32c, pre, ws->b32, ws->x32, ws->r32, ws->p32, ws->pb32, ws->q32, ws->z32, c->opt.inner_tol,
                                    maxit, 1.0, 1);
                else
                    solve_gmres<float>(F, A32, A32i, AP32, P32, pre, ws->b32, ws->x32, ws->V32, ws->w32, ws->z32, ws->t32,
@@ -1304,7 +1146,7 @@ int solver_setup(stdg_ctx* c) {
                                ws->owned.push_back((void*)(ptr)); } while (0)
     ALLOC(ws->sc, sizeof(DevScalars));
     ALLOC(ws->ss, sizeof(ShotScalars) * ws->ns);
-    ALLOC(ws->partials, sizeof(double) * (kMaxRestart + 2) * ws->G * ws->ns);
+    ALLOC(ws->partials, sizeof(double) * (kMaxRestart + 2) * std::max(ws->G * ws->ns, (unsigned)(4 * c->n_sm)));
     ALLOC(ws->done, sizeof(unsigned) * (ws->ns + 1));
     ALLOC(ws->dparams, sizeof(double) * 4);
     ALLOC(c->d_b, sizeof(double) * n);
@@ -1312,6 +1154,8 @@ int solver_setup(stdg_ctx* c) {
     ALLOC(ws->w, sizeof(double) * n);
     ALLOC(ws->r, sizeof(double) * n);
     ws->ldv = (n + 63) / 64 * 64;   // 16-byte aligned basis columns for vector loads
+    if (cn && !mixed && pre) ALLOC(ws->pb, sizeof(double) * n);
+    if (cn && mixed && pre) ALLOC(ws->pb32, sizeof(float) * n);
     if (cn && !mixed) { ALLOC(ws->p, sizeof(double) * n); ALLOC(ws->q, sizeof(double) * n); }
     if (!cn && !mixed) ALLOC(ws->V, sizeof(double) * ws->ldv * (ws->m + 1));
     if (pre && !mixed) { ALLOC(ws->z, sizeof(double) * n); if (!cn) ALLOC(ws->t, sizeof(double) * n); }

@@ -71,7 +71,8 @@ int build_host_mesh(int dim, int64_t n_vert, const double* xyz, int64_t n_elem, 
 int64_t locate_point(const HostMesh& m, const double* x, double* x_local);
 
 // Krylov workspace and step graph state live in the context.
-struct Scalars;   // device-side solver scalars (defined in solver.cu)
+struct DevScalars;    // device-side solver scalars (krylov.h)
+struct ShotScalars;
 
 }  // namespace stdg
 
@@ -294,6 +295,14 @@ bool launch_pre2_local_mma(stdg_ctx* c, const float* r, const int* ridx, int64_t
                            int nshots, cudaError_t* e);
 // (re)build the dt-dependent preconditioner blocks when dt changes (capi.cu)
 int precond_for_dt(stdg_ctx* c, double dt);
+
+// cg_fused.cu: CG of the block-Jacobi preconditioned Crank-Nicolson system (one shot): two kernels an
+// iteration, or all iterations of a small system in one cluster; p and pb hold the search directions of even and odd iterations
+bool cg_fused_applies(const stdg_ctx* c, int nshots, bool fp32);
+cudaError_t launch_cg_fused(stdg_ctx* c, double dt, double* x, double* r, double* z, double* p, double* pb, double* q,
+                            DevScalars* sc, ShotScalars* ss, double* part, unsigned* done, cudaGraphConditionalHandle h, int use_h);
+cudaError_t launch_cg_fused(stdg_ctx* c, double dt, float* x, float* r, float* z, float* p, float* pb, float* q, DevScalars* sc,
+                            ShotScalars* ss, double* part, unsigned* done, cudaGraphConditionalHandle h, int use_h);
 
 // solver.cu
 int solver_setup(stdg_ctx* c);

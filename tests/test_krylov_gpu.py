@@ -14,6 +14,9 @@ CASES = [  # cells, p, p_gamma, scheme, shots, restart, preconditioner, precisio
     (2, 1, 0, "cn", 1, 30, 1, "fp64"),
     (3, 1, 0, "cn", 3, 30, 1, "mixed"),
     (3, 2, 0, "cn", 2, 30, 0, "fp64"),
+    (4, 2, 0, "cn", 1, 30, 1, "mixed"),
+    (3, 3, 0, "cn", 1, 30, 1, "fp64"),
+    (2, 4, 0, "cn", 1, 30, 1, "mixed"),
     (2, 1, 1, "stdg", 1, 2, 1, "fp64"),
     (3, 2, 1, "stdg", 3, 15, 1, "fp64"),
     (3, 2, 1, "stdg", 3, 16, 1, "mixed"),
@@ -49,3 +52,24 @@ def test_small_and_unaligned_solves(cells, p, pg, scheme, shots, restart, pre, p
     for k, sim in enumerate(sims):
         v, _ = s.get_state(k)
         assert rel_l2(v, sim.v_tr) < tol
+
+
+@pytest.mark.parametrize("p,precision", [(1, "fp64"), (2, "mixed"), (3, "fp64"), (1, "mixed")])
+def test_crank_nicolson_3d(p, precision):
+    need_gpu()
+    from paper_1802_04516_gb300.binding import Solver
+    xyz, ev, per = synth.tet_kuhn(1 if p == 3 else 2, 1.0, periodic=False, jitter=0.1, seed=4)
+    rng = np.random.default_rng(9)
+    n = ev.shape[0]
+    w = synth.Workload("cg3", 3, xyz, ev, per, rng.uniform(1, 2, n), rng.uniform(.5, 1, n), rng.uniform(.8, 1.2, n),
+                       p=p, p_gamma=0, scheme="cn", dt=0.05, n_steps=3, h=0.5)
+    s = Solver(3, p, 0, scheme="cn", precision=precision, rel_tol=1e-13 if precision == "fp64" else 1e-12, max_iters=20000)
+    s.set_mesh(xyz, ev, per)
+    s.set_material(w.lam, w.mu, w.rho)
+    sim = oracle_sim(w)
+    v, sig = rng.normal(size=sim.v_tr.shape), rng.normal(size=sim.sig_tr.shape)
+    sim.set_state(v, sig)
+    s.set_state(v, sig)
+    s.step(w.dt, 3)
+    sim.step(3)
+    assert rel_l2(s.get_state()[0], sim.v_tr) < (1e-10 if precision == "fp64" else 1e-8)
