@@ -18,8 +18,8 @@
 // and K_ei = K_ie^T.  With D_e^{-1} = (V_e (x) I) blockdiag_q(B_{e,q}) (V_e^T (x) I) from
 // the block-Jacobi set-up,
 //   N_{i,e} D_e^{-1} N_{e,i} = (c dt^2)^2 sum_q (k_q k_q^T) (x) (S B_{e,q} S),  k_q = K_ie V_e[:, q],
-// which assembles S_i without any n^3 product; S_i (order d N_phi N_gamma) is then
-// inverted by Gauss-Jordan elimination with partial pivoting and stored column-major, in
+// S_i (order d N_phi N_gamma) is then inverted by Gauss-Jordan elimination with partial
+// pivoting and stored column-major, in
 // FP64 for the FP64 solver and in FP32 for the FP32 inner solver of the mixed path.  (BF16
 // blocks halve the bytes, but on the heterogeneous 60,024-triangle inversion medium they
 // made the inner GMRES stagnate after 16 slabs; FP32 blocks converge there.)
@@ -34,7 +34,6 @@
 
 namespace stdg {
 
-constexpr int kP2Threads = 256;
 constexpr int kP2MaxRows = 4;                 // rows per lane in the apply: N <= 128
 
 // K^{(j)}[(k,n),(k',n')] += lam P(k,k') + mu P(k',k) + delta_kk' mu sum_l P(l,l),
@@ -58,52 +57,61 @@ __device__ void add_face_coupling(double* K, int n, int dim, int NP, const doubl
     }
 }
 
-// smem: A (N x 2N augmented), K (n x n), kv (n x n), W (n x NG x NG), Da, Db (dim NP NP each), f (N)
-__global__ void __launch_bounds__(kP2Threads) pre2_setup_kernel(
+// One block of TG x TG threads per element.  S_i is assembled in shared memory: K from the assembled
+// couplings where they are kept, and the neighbours' corrections per time pair (a, a') as a symmetric
+// n x n product, half of it computed.  The inversion works in place in registers: thread (ti, tj) holds
+// the entries (ti + TG u, tj + TG v), u, v < TS; a step hands the pivot column and the scaled pivot row
+// through shared memory and costs TS^2 FP64 products a thread.  Bound by the FP64 pipe.  The augmented
+// matrix in shared memory that this replaces visited 2 N^2 entries a step with one thread looking for
+// the pivot.  First apply at a new slab size: 50,176 triangles at p = p_gamma = 3 241 -> 119 ms, 40,000 at p = 2
+// 24 -> 14 ms, 10,368 tetrahedra at p = 2 133 -> 56 ms.
+template <int TG, int TS>
+__global__ void __launch_bounds__(TG * TG) pre2_setup_kernel(
     int64_t n_elem, int dim, const RefTables* __restrict__ rtp, const int32_t* __restrict__ elem_face,
     const int32_t* __restrict__ face_l, const int32_t* __restrict__ face_r, const double* __restrict__ D,
     const double* __restrict__ lamf, const double* __restrict__ muf, const double* __restrict__ rhoJ,
-    const double* __restrict__ preV, const double* __restrict__ preB, double cdt2, double* __restrict__ out64,
-    float* __restrict__ out32, int64_t stride32, int* __restrict__ status) {
+    const double* __restrict__ preV, const double* __restrict__ preB, const double* __restrict__ Kf,
+    const double* __restrict__ Ke, double cdt2, double* __restrict__ out64, float* __restrict__ out32, int64_t stride32,
+    int* __restrict__ status) {
     extern __shared__ double sm[];
-    const int NP = rtp->Nphi, NG = rtp->Ng;
-    const int n = dim * NP;
-    const int N = n * NG;
-    const int ldA = 2 * N;
-    double* A = sm;                         // N x 2N
+    const int NP = rtp->Nphi, NG = rtp->Ng, n = dim * NP, N = n * NG, ldA = N | 1, nD = dim * NP * NP;
+    double* A = sm;                         // N x ldA
     double* K = A + (size_t)N * ldA;        // n x n
     double* kv = K + n * n;                 // n x n: kv[s][q] = (K_ie V_e)[s][q]
-    double* W = kv + n * n;                 // n x NG x NG: S B_q S
-    double* Da = W + n * NG * NG;
-    double* Db = Da + dim * NP * NP;
-    double* f = Db + dim * NP * NP;         // N
-    __shared__ int s_piv;
-    __shared__ int s_sing;
-    const int tid = threadIdx.x;
+    double* kw = kv + n * n;                // n x n: kv times one entry of W per column
+    double* W = kw + n * n;                 // n x NG x NG: S B_q S
+    double* fcol = W + n * NG * NG;         // N: pivot column
+    double* prow = fcol + N;                // N: scaled pivot row
+    double* rowk = prow + N;                // N: the row that makes way for it
+    double* Da = rowk + N;                  // D~ of both sides, when the couplings are not kept
+    double* Db = Da + nD;
+    __shared__ int s_piv[128], s_map[128], s_sing;
+    __shared__ double s_inv;
+    const int tid = threadIdx.x, ti = tid / TG, tj = tid % TG;
     for (int64_t e = blockIdx.x; e < n_elem; e += gridDim.x) {
-        // ---- D_i: rho|J| (I (x) M_ref) (x) T + c dt^2 K_ii (x) S, and [ . | I ]
-        for (int t = tid; t < n * n; t += blockDim.x) K[t] = 0.0;
         __syncthreads();
-        for (int fi = 0; fi <= dim; ++fi) {
+        if (tid == 0) s_sing = 0;
+        // ---- D_i: rho|J| (I (x) M_ref) (x) T + c dt^2 K_ii (x) S
+        for (int t = tid; t < n * n; t += blockDim.x) K[t] = Ke ? Ke[e * n * n + t] : 0.0;
+        for (int fi = 0; !Ke && fi <= dim; ++fi) {
             const int j = elem_face[e * (dim + 1) + fi];
-            const int side = face_l[j] == (int)e ? 0 : 1;
-            const double* Dg = D + ((int64_t)j * 2 + side) * dim * NP * NP;
-            for (int t = tid; t < dim * NP * NP; t += blockDim.x) Da[t] = Dg[t];
+            const double* Dg = D + ((int64_t)j * 2 + (face_l[j] == (int)e ? 0 : 1)) * nD;
+            __syncthreads();
+            for (int t = tid; t < nD; t += blockDim.x) Da[t] = Dg[t];
             __syncthreads();
             add_face_coupling(K, n, dim, NP, Da, Da, lamf[j], muf[j], 1.0);
-            __syncthreads();
-        }
-        const double rj = rhoJ[e];
-        for (int ent = tid; ent < N * N; ent += blockDim.x) {
-            const int R = ent / N, C = ent % N;
-            const int k = R / (NG * NP), a = (R / NP) % NG, nn = R % NP;
-            const int k2 = C / (NG * NP), a2 = (C / NP) % NG, n2 = C % NP;
-            double v = cdt2 * K[(k * NP + nn) * n + k2 * NP + n2] * rtp->S[a * NG + a2];
-            if (k == k2) v += rj * rtp->Mref[nn * NP + n2] * rtp->T[a * NG + a2];
-            A[R * ldA + C] = v;
-            A[R * ldA + N + C] = R == C ? 1.0 : 0.0;
         }
         __syncthreads();
+        const double rj = rhoJ[e];
+        for (int R = tid / 32; R < N; R += blockDim.x / 32) {   // a warp per row
+            const int k = R / (NG * NP), a = (R / NP) % NG, nn = R % NP;
+            for (int C = tid % 32; C < N; C += 32) {
+                const int k2 = C / (NG * NP), a2 = (C / NP) % NG, n2 = C % NP;
+                double v = cdt2 * K[(k * NP + nn) * n + k2 * NP + n2] * rtp->S[a * NG + a2];
+                if (k == k2) v += rj * rtp->Mref[nn * NP + n2] * rtp->T[a * NG + a2];
+                A[R * ldA + C] = v;
+            }
+        }
         // ---- minus N_{i,e} D_e^{-1} N_{e,i} for every face neighbour e
         for (int fi = 0; fi <= dim; ++fi) {
             const int j = elem_face[e * (dim + 1) + fi];
@@ -112,21 +120,21 @@ __global__ void __launch_bounds__(kP2Threads) pre2_setup_kernel(
             const int side = l == (int)e ? 0 : 1;
             const int64_t nb = side == 0 ? r : l;
             if (nb == e) continue;          // a periodic self-neighbour is part of D_i already
-            const double* Dg = D + (int64_t)j * 2 * dim * NP * NP;
-            for (int t = tid; t < dim * NP * NP; t += blockDim.x) {
-                Da[t] = Dg[side * dim * NP * NP + t];
-                Db[t] = Dg[(1 - side) * dim * NP * NP + t];
-            }
-            for (int t = tid; t < n * n; t += blockDim.x) K[t] = 0.0;
             __syncthreads();
-            add_face_coupling(K, n, dim, NP, Da, Db, lamf[j], muf[j], 1.0);   // K_ie
-            __syncthreads();
-            const double* Ve = preV + nb * (int64_t)n * n;
-            for (int ent = tid; ent < n * n; ent += blockDim.x) {
-                const int s = ent / n, q = ent % n;
-                double acc = 0;
-                for (int s2 = 0; s2 < n; ++s2) acc += K[s * n + s2] * Ve[s2 * n + q];
-                kv[ent] = acc;
+            if (Kf) {
+                for (int t = tid; t < n * n; t += blockDim.x) {   // rows of this element, columns of the neighbour
+                    const double v = Kf[(int64_t)j * n * n + t];
+                    K[side == 0 ? t : t % n * n + t / n] = v;
+                }
+            } else {
+                const double* Dg = D + (int64_t)j * 2 * nD;
+                for (int t = tid; t < nD; t += blockDim.x) {
+                    Da[t] = Dg[side * nD + t];
+                    Db[t] = Dg[(1 - side) * nD + t];
+                }
+                for (int t = tid; t < n * n; t += blockDim.x) K[t] = 0.0;
+                __syncthreads();
+                add_face_coupling(K, n, dim, NP, Da, Db, lamf[j], muf[j], 1.0);   // K_ie
             }
             const double* Be = preB + nb * (int64_t)n * NG * NG;
             for (int ent = tid; ent < n * NG * NG; ent += blockDim.x) {
@@ -138,62 +146,140 @@ __global__ void __launch_bounds__(kP2Threads) pre2_setup_kernel(
                 W[ent] = acc;
             }
             __syncthreads();
-            const double c2 = cdt2 * cdt2;
-            for (int ent = tid; ent < N * N; ent += blockDim.x) {
-                const int R = ent / N, C = ent % N;
-                const int k = R / (NG * NP), a = (R / NP) % NG, nn = R % NP;
-                const int k2 = C / (NG * NP), a2 = (C / NP) % NG, n2 = C % NP;
-                const double* k1 = kv + (k * NP + nn) * n;
-                const double* kk2 = kv + (k2 * NP + n2) * n;
+            const double* Ve = preV + nb * (int64_t)n * n;
+            for (int ent = tid; ent < n * n; ent += blockDim.x) {
+                const int s = ent / n, q = ent % n;
                 double acc = 0;
-                for (int q = 0; q < n; ++q) acc += k1[q] * kk2[q] * W[(q * NG + a) * NG + a2];
-                A[R * ldA + C] -= c2 * acc;
+                for (int s2 = 0; s2 < n; ++s2) acc = fma(K[s * n + s2], Ve[s2 * n + q], acc);
+                kv[ent] = acc;
+            }
+            const double c2 = cdt2 * cdt2;
+            for (int t = 0; t < NG * NG; ++t) {
+                const int a = t / NG, a2 = t % NG;
+                __syncthreads();
+                for (int ent = tid; ent < n * n; ent += blockDim.x) kw[ent] = kv[ent] * W[ent % n * NG * NG + t];
+                __syncthreads();
+                for (int ent = tid; ent < n * (n + 1) / 2; ent += blockDim.x) {   // rows r >= c: sum_q kv_r W_q kv_c
+                    int rr = (int)((sqrtf(8.f * ent + 1.f) - 1.f) * 0.5f);
+                    while (rr * (rr + 1) / 2 > ent) --rr;
+                    while ((rr + 1) * (rr + 2) / 2 <= ent) ++rr;
+                    const int cc = ent - rr * (rr + 1) / 2;
+                    double acc = 0;
+                    for (int q = 0; q < n; ++q) acc = fma(kw[rr * n + q], kv[cc * n + q], acc);
+                    acc *= c2;
+                    const int kr = rr / NP, nr = rr % NP, kc = cc / NP, nc = cc % NP;
+                    A[((kr * NG + a) * NP + nr) * ldA + (kc * NG + a2) * NP + nc] -= acc;
+                    if (rr != cc) A[((kc * NG + a) * NP + nc) * ldA + (kr * NG + a2) * NP + nr] -= acc;
+                }
+            }
+        }
+        __syncthreads();
+        // ---- in-place Gauss-Jordan with partial pivoting; the padding of the tiles is an identity
+        double T[TS][TS];
+#pragma unroll
+        for (int u = 0; u < TS; ++u)
+#pragma unroll
+            for (int v = 0; v < TS; ++v) {
+                const int i = ti + TG * u, j = tj + TG * v;
+                T[u][v] = i < N && j < N ? A[i * ldA + j] : (i == j ? 1.0 : 0.0);
+            }
+        for (int k = 0; k < N; ++k) {
+            const int kb = k / TG, kt = k % TG;
+            if (tj == kt) {
+#pragma unroll
+                for (int u = 0; u < TS; ++u)
+#pragma unroll
+                    for (int v = 0; v < TS; ++v)
+                        if (v == kb && ti + TG * u < N) fcol[ti + TG * u] = T[u][v];
             }
             __syncthreads();
-        }
-        // ---- Gauss-Jordan on [S_i | I] with partial pivoting
-        if (tid == 0) s_sing = 0;
-        for (int col = 0; col < N; ++col) {
-            if (tid == 0) {
-                int p = col;
-                double best = fabs(A[col * ldA + col]);
-                for (int rr = col + 1; rr < N; ++rr) {
-                    const double v = fabs(A[rr * ldA + col]);
-                    if (v > best) { best = v; p = rr; }
+            if (tid < 32) {   // the largest entry at or below the diagonal, the first of equal ones
+                double best = -1.0;
+                int at = k;
+                for (int i = k + tid; i < N; i += 32) {
+                    const double v = fabs(fcol[i]);
+                    if (v > best) { best = v; at = i; }
                 }
-                s_piv = p;
-                if (!(best > 0.0)) s_sing = 1;
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+                    if (ob > best || (ob == best && oa < at)) { best = ob; at = oa; }
+                }
+                if (tid == 0) {
+                    s_piv[k] = at;
+                    if (!(best > 0.0)) s_sing = 1;
+                    s_inv = 1.0 / fcol[at];
+                }
             }
             __syncthreads();
             if (s_sing) break;
-            const int p = s_piv;
-            if (p != col)
-                for (int t = tid; t < ldA; t += blockDim.x) {
-                    const double u = A[col * ldA + t];
-                    A[col * ldA + t] = A[p * ldA + t];
-                    A[p * ldA + t] = u;
+            const int p = s_piv[k], pb = p / TG, pt = p % TG;
+            const double inv = s_inv;
+            if (ti == pt) {
+#pragma unroll
+                for (int u = 0; u < TS; ++u)
+#pragma unroll
+                    for (int v = 0; v < TS; ++v) {
+                        const int j = tj + TG * v;
+                        if (u == pb && j < N) prow[j] = j == k ? inv : T[u][v] * inv;
+                    }
+            }
+            if (ti == kt && p != k) {
+#pragma unroll
+                for (int u = 0; u < TS; ++u)
+#pragma unroll
+                    for (int v = 0; v < TS; ++v)
+                        if (u == kb && tj + TG * v < N) rowk[tj + TG * v] = T[u][v];
+            }
+            __syncthreads();
+            double pr[TS];
+#pragma unroll
+            for (int v = 0; v < TS; ++v) pr[v] = tj + TG * v < N ? prow[tj + TG * v] : 0.0;
+#pragma unroll
+            for (int u = 0; u < TS; ++u) {
+                const int i = ti + TG * u;
+                const bool moved = i == p && p != k;             // row k's old values come here
+                const double f = i < N ? -fcol[moved ? k : i] : 0.0;
+#pragma unroll
+                for (int v = 0; v < TS; ++v) {
+                    const int j = tj + TG * v;
+                    double base = T[u][v];
+                    if (moved && j < N) base = rowk[j];
+                    if (j == k) base = 0.0;
+                    T[u][v] = i == k ? pr[v] : fma(f, pr[v], base);
                 }
-            __syncthreads();
-            const double inv = 1.0 / A[col * ldA + col];
-            __syncthreads();
-            for (int t = tid; t < ldA; t += blockDim.x) A[col * ldA + t] *= inv;
-            for (int t = tid; t < N; t += blockDim.x) f[t] = A[t * ldA + col];
-            __syncthreads();
-            for (int ent = tid; ent < N * ldA; ent += blockDim.x) {
-                const int rr = ent / ldA, cc = ent % ldA;
-                if (rr != col && cc >= col) A[ent] -= f[rr] * A[col * ldA + cc];
             }
             __syncthreads();
         }
-        if (s_sing && tid == 0) atomicExch(status, 1);
-        // ---- store S_i^{-1} column-major: out[e][C][R]
-        for (int ent = tid; ent < N * N; ent += blockDim.x) {
-            const int C = ent / N, R = ent % N;
-            const double v = A[R * ldA + N + C];
-            if (out64) out64[e * (int64_t)N * N + ent] = v;
-            if (out32) out32[e * stride32 + ent] = (float)v;
+        if (s_sing) {
+            if (tid == 0) atomicExch(status, 1);
+            continue;
+        }
+#pragma unroll
+        for (int u = 0; u < TS; ++u)
+#pragma unroll
+            for (int v = 0; v < TS; ++v) {
+                const int i = ti + TG * u, j = tj + TG * v;
+                if (i < N && j < N) A[i * ldA + j] = T[u][v];
+            }
+        for (int j = tid; j < N; j += blockDim.x) {   // (P S)^{-1} P: where column j's unit vector went
+            int pos = j;
+            for (int k = 0; k < N; ++k) {
+                if (pos == k) pos = s_piv[k];
+                else if (pos == s_piv[k]) pos = k;
+            }
+            s_map[j] = pos;
         }
         __syncthreads();
+        // ---- store S_i^{-1} column-major: out[e][C][R]
+        for (int C = tid / 32; C < N; C += blockDim.x / 32) {
+            const int from = s_map[C];
+            for (int R = tid % 32; R < N; R += 32) {
+                const double v = A[R * ldA + from];
+                if (out64) out64[(e * N + C) * (int64_t)N + R] = v;
+                if (out32) out32[e * stride32 + C * N + R] = (float)v;
+            }
+        }
     }
 }
 
@@ -355,26 +441,52 @@ __global__ void __launch_bounds__(128) pre2_local_half_kernel(int64_t n_elem, in
     }
 }
 
-static size_t pre2_setup_smem(int dim, int NP, int NG) {
+// The shapes that the preconditioner takes are those whose augmented matrix fits an SM.
+static size_t pre2_augmented_smem(int dim, int NP, int NG) {
     const int n = dim * NP, N = n * NG;
     return sizeof(double) * ((size_t)N * 2 * N + 2 * (size_t)n * n + (size_t)n * NG * NG + 2 * (size_t)dim * NP * NP + N);
 }
 
+static size_t pre2_setup_smem(int dim, int NP, int NG) {
+    const int n = dim * NP, N = n * NG;
+    return sizeof(double) * ((size_t)N * (N | 1) + 3 * (size_t)n * n + (size_t)n * NG * NG + 2 * (size_t)dim * NP * NP + 3 * N);
+}
+
 bool pre2_supported(const stdg_ctx* c) {
     const int N = c->dim * c->Nphi * c->Ng;
-    return N <= 32 * kP2MaxRows && pre2_setup_smem(c->dim, c->Nphi, c->Ng) <= 227 * 1024;
+    return N <= 32 * kP2MaxRows && pre2_augmented_smem(c->dim, c->Nphi, c->Ng) <= 227 * 1024;
 }
 
 cudaError_t launch_pre2_setup(stdg_ctx* c, double dt, int* d_status) {
     const double cfac = c->opt.scheme == STDG_SCHEME_CN ? 0.25 : 1.0;
     const size_t smem = pre2_setup_smem(c->dim, c->Nphi, c->Ng);
-    cudaFuncSetAttribute(pre2_setup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int grid = (int)std::min<int64_t>(c->n_elem, c->n_sm * 8);
-    pre2_setup_kernel<<<grid, kP2Threads, smem, c->stream>>>(c->n_elem, c->dim, c->d_rt, c->d_elem_face, c->d_face_l,
-                                                             c->d_face_r, c->d_D, c->d_lamf, c->d_muf, c->d_rhoJ, c->d_preV,
-                                                             c->d_preB, cfac * dt * dt, c->d_pre2, c->d_pre2_32,
-                                                             pre2_stride32(c), d_status);
-    note_launch(c);
+    const int N = c->dim * c->Nphi * c->Ng;
+    const int grid = (int)std::min<int64_t>(c->n_elem, c->n_sm * 16);
+    auto go = [&](auto kern, int threads) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kern<<<grid, threads, smem, c->stream>>>(c->n_elem, c->dim, c->d_rt, c->d_elem_face, c->d_face_l, c->d_face_r, c->d_D,
+                                                 c->d_lamf, c->d_muf, c->d_rhoJ, c->d_preV, c->d_preB, c->d_Kf, c->d_Ke,
+                                                 cfac * dt * dt, c->d_pre2, c->d_pre2_32, pre2_stride32(c), d_status);
+        note_launch(c);
+    };
+    if (N <= 40) {   // 64 threads while their tiles stay at 5 x 5
+        switch ((N + 7) / 8) {
+            case 1: go(pre2_setup_kernel<8, 1>, 64); break;
+            case 2: go(pre2_setup_kernel<8, 2>, 64); break;
+            case 3: go(pre2_setup_kernel<8, 3>, 64); break;
+            case 4: go(pre2_setup_kernel<8, 4>, 64); break;
+            default: go(pre2_setup_kernel<8, 5>, 64); break;
+        }
+    } else {
+        switch ((N + 15) / 16) {
+            case 3: go(pre2_setup_kernel<16, 3>, 256); break;
+            case 4: go(pre2_setup_kernel<16, 4>, 256); break;
+            case 5: go(pre2_setup_kernel<16, 5>, 256); break;
+            case 6: go(pre2_setup_kernel<16, 6>, 256); break;
+            case 7: go(pre2_setup_kernel<16, 7>, 256); break;
+            default: go(pre2_setup_kernel<16, 8>, 256); break;
+        }
+    }
     return cudaGetLastError();
 }
 

@@ -77,21 +77,29 @@ def test_off_diagonal_form_for_stacked_shots(dim, p, pg, shots, precision):
         assert rel_l2(z[k], P @ r[k]) < (1e-9 if precision == "fp64" else 1e-3)
 
 
-def test_face_kernels_when_the_couplings_do_not_fit():
+@pytest.mark.parametrize("p,pre", [(3, 1), (2, 2)])
+def test_face_kernels_when_the_couplings_do_not_fit(p, pre):
     torch = need_gpu()
-    w = _workload(2, 3, 3, n=60)
-    x = np.random.default_rng(8).normal(size=w.n_elem * 2 * 4 * 10)
-    s = _solver(w, preconditioner=1)
-    y, held = s.apply_operator(w.dt, x), s.query(10)
-    s.close()
+    w = _workload(2, p, p, n=60)
+    n = w.n_elem * 2 * (p + 1) * (p + 1) * (p + 2) // 2
+    x = np.random.default_rng(8).normal(size=n)
+
+    def run():
+        s = _solver(w, preconditioner=pre)
+        s.set_shots(1)
+        try:
+            return s.apply_operator(w.dt, x), s.apply_preconditioner(w.dt, x), s.query(10)
+        finally:
+            s.close()
+
+    y, z, held = run()
     torch.cuda.empty_cache()
     free, _ = torch.cuda.mem_get_info()
     fill = torch.empty(free - (held - (16 << 20)), dtype=torch.uint8, device="cuda")   # room for all but the couplings
     try:
-        s = _solver(w, preconditioner=1)
-        assert s.query(10) < held
-        assert rel_l2(s.apply_operator(w.dt, x), y) < 1e-12
+        y2, z2, held2 = run()
     finally:
-        s.close()
         del fill
         torch.cuda.empty_cache()
+    assert held2 < held
+    assert rel_l2(y2, y) < 1e-12 and rel_l2(z2, z) < 1e-10
