@@ -80,7 +80,7 @@ def test_off_diagonal_form_for_stacked_shots(dim, p, pg, shots, precision):
 @pytest.mark.parametrize("p,pre", [(3, 1), (2, 2)])
 def test_face_kernels_when_the_couplings_do_not_fit(p, pre):
     torch = need_gpu()
-    w = _workload(2, p, p, n=60)
+    w = _workload(2, p, p, n=120)
     n = w.n_elem * 2 * (p + 1) * (p + 1) * (p + 2) // 2
     x = np.random.default_rng(8).normal(size=n)
 
@@ -88,16 +88,18 @@ def test_face_kernels_when_the_couplings_do_not_fit(p, pre):
         s = _solver(w, preconditioner=pre)
         s.set_shots(1)
         try:
-            return s.apply_operator(w.dt, x), s.apply_preconditioner(w.dt, x), s.query(10)
+            couplings = 8 * (s.n_face + s.n_elem) * (w.dim * s.Nphi) ** 2
+            return s.apply_operator(w.dt, x), s.apply_preconditioner(w.dt, x), s.query(10), couplings
         finally:
             s.close()
 
-    y, z, held = run()
+    y, z, held, couplings = run()
     torch.cuda.empty_cache()
     free, _ = torch.cuda.mem_get_info()
-    fill = torch.empty(free - (held - (16 << 20)), dtype=torch.uint8, device="cuda")   # room for all but the couplings
+    # all but the couplings fits: half their size is left for the granularity of the allocator
+    fill = torch.empty(free - (held - couplings // 2), dtype=torch.uint8, device="cuda")
     try:
-        y2, z2, held2 = run()
+        y2, z2, held2, _ = run()
     finally:
         del fill
         torch.cuda.empty_cache()
