@@ -73,3 +73,28 @@ def test_crank_nicolson_3d(p, precision):
     s.step(w.dt, 3)
     sim.step(3)
     assert rel_l2(s.get_state()[0], sim.v_tr) < (1e-10 if precision == "fp64" else 1e-8)
+
+
+@pytest.mark.parametrize("nx,ny,p,precision", [  # one cluster holds 1,360 triangles at p = 1 and 672 at p = 2
+    (20, 34, 1, "fp64"), (21, 33, 1, "fp64"), (21, 33, 1, "mixed"), (40, 31, 1, "fp64"),
+    (16, 21, 2, "mixed"), (17, 21, 2, "mixed"), (17, 21, 2, "fp64")])
+def test_crank_nicolson_around_the_cluster_limit(nx, ny, p, precision):
+    need_gpu()
+    from paper_1802_04516_gb300.binding import Solver
+    xyz, ev, per = synth.tri_grid(nx, ny, 1.0, 1.0, periodic=False, jitter=0.2, seed=6)
+    rng = np.random.default_rng(12)
+    n = ev.shape[0]
+    w = synth.Workload("krylov", 2, xyz, ev, per, rng.uniform(1, 2, n), rng.uniform(.5, 1, n), rng.uniform(.8, 1.2, n),
+                       p=p, p_gamma=0, scheme="cn", dt=0.02, n_steps=2, h=1.0 / nx)
+    sim = oracle_sim(w)
+    v, sig = rng.normal(size=sim.v_tr.shape), rng.normal(size=sim.sig_tr.shape)
+    sim.set_state(v, sig)
+    sim.step(2)
+    s = Solver(2, p, 0, scheme="cn", precision=precision, rel_tol=1e-13 if precision == "fp64" else 1e-12, max_iters=20000,
+               preconditioner=1)
+    s.set_mesh(xyz, ev, per)
+    s.set_material(w.lam, w.mu, w.rho)
+    s.set_state(v, sig)
+    s.step(w.dt, 2)
+    out, _ = s.get_state()
+    assert rel_l2(out, sim.v_tr) < (1e-10 if precision == "fp64" else 1e-8)
