@@ -112,6 +112,10 @@ int stdg_set_mesh(stdg_ctx* ctx, int64_t n_vert, const double* xyz, int64_t n_el
  * constant per element; E_j constant per dual cell, the sub-cell-measure-weighted mean
  * of its two elements.  Requires lambda >= 0, mu > 0, rho > 0, all finite (else
  * STDG_EINVAL); STDG_ESTATE before stdg_set_mesh.  Also sets up the preconditioner. */
+/* The operator's element couplings are laid out on the device with the medium, (d N_phi)^2 FP64
+ * values per face and per element plus FP32 copies in mixed precision, where they take no more than a third of the free
+ * memory; they are given back when a later allocation of the context needs the room, and the
+ * operator then runs from the face blocks. */
 int stdg_set_material(stdg_ctx* ctx, const double* lambda, const double* mu, const double* rho);
 
 /* Per-element time scale alpha (n_elem values, > 0, finite), for disconnected parts of one
@@ -271,7 +275,7 @@ int stdg_apply_preconditioner(stdg_ctx* ctx, double dt, const double* r, double*
  * velocity values per slab, canonical layout), on device buffers owned by the caller (r_dev
  * and z_dev distinct), slab size dt.  fp32 = 0: the FP64 preconditioner of the FP64 solver;
  * fp32 != 0 (mixed-precision contexts only): the FP32 one of the inner solve -- for the stencil
- * preconditioner with several shots and d N_phi N_gamma = 36, its element-local step runs on
+ * preconditioner with more than 24 shots and d N_phi N_gamma = 36, its element-local step runs on
  * the tensor cores (kind::tf32 with S^{-1} rounded to TF32 and the vector split into two TF32
  * terms).  Appendix A, Eq. pre1 (Pre1) or Eqs. APPRE1-APPRE2 (Pre2).  Synchronises the stream;
  * STDG_ESTATE without a preconditioner or shots, STDG_ECUDA if a bounded wait gave up. */

@@ -795,9 +795,9 @@ cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, dou
 }
 
 // FP32: couplings or face kernels.  The two shapes with a tiled single-shot face kernel keep it, and
-// no FP32 couplings: 3D at p = p_gamma = 2, where a face's couplings are 1.5 times its D~ (217 us
-// against 310 us with the mass term on 82,944 tetrahedra), and 2D at p = p_gamma = 3, where they are
-// faster (264 against 325 us on 200,704 triangles) but move the mixed slab of the sliver mesh by more
+// no FP32 couplings: 3D at p = p_gamma = 2, where a face's couplings are 1.5 times its D~ (310 us
+// against 181 + 12 us, face and mass kernel, on 82,944 tetrahedra), and 2D at p = p_gamma = 3, where they
+// are little faster (264 against 253 + 22 us, cold, on 200,704 triangles) and move the mixed slab of the sliver mesh by more
 // than two runs differ (its inner residual is met by a different iterate; single velocities by 3e-7).
 // Elsewhere they win at every size (2D p = 2: 117 against 238 us on 200,704 triangles).
 // In 3D with one time node D~ is read for few products and the couplings only win while they stay in
