@@ -30,9 +30,10 @@ struct Coupling {
     static constexpr int RPT = BOTH ? 2 : 1, TPE = N / RPT;   // rows per thread, threads per element
     static constexpr int NGP = NG <= 2 ? NG : (NG <= 4 ? 4 : 6);          // row stride of the staged values
     static constexpr int VJ = !BOTH || SC > 1 ? 2 : (N % 10 == 0 ? 10 : 6);   // columns loaded together
-    static constexpr int CH = !BOTH ? N : (N % 10 == 0 ? 10 : 6);         // columns summed before they join the total
-    static constexpr bool NEST = BOTH && N > 20;                          // the chunks of a block join a sum of its own
-    static_assert(N % CH == 0 && CH % VJ == 0, "chunks of whole loads");
+    static constexpr int BL = !BOTH ? N : (N % 10 == 0 ? 10 : 6);         // columns per turn of the loop
+    // FP32: columns summed before they join the total, and the joins are compensated (Kahan 1965)
+    static constexpr int CH = !BOTH || SC > 1 ? BL : BL / 2;
+    static_assert(N % BL == 0 && BL % VJ == 0 && (CH == BL || (VJ == BL && VJ % CH == 0)), "chunks of whole loads");
     static_assert(N % 2 == 0, "d N_phi is even for every supported order");
     __host__ __device__ static constexpr int slots(bool own) { return FACES + (own ? 1 : 0); }
     static size_t smem(int EB, bool own) { return sizeof(R) * (size_t)SC * slots(own) * EB * N * NGP; }
@@ -103,13 +104,16 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                 for (int a = 0; a < NG; ++a) bs[r][a] = base[(int64_t)s0 * nvec + (e0 + le) * NV + (k * NG + a) * NP + nn];
             }
         }
-        R acc[RPT][SC][NG];
+        R acc[RPT][SC][NG], lost[C::BOTH ? RPT : 1][C::BOTH ? SC : 1][C::BOTH ? NG : 1];   // totals, what their last join rounded away
 #pragma unroll
         for (int r = 0; r < RPT; ++r)
 #pragma unroll
             for (int c = 0; c < SC; ++c)
 #pragma unroll
-                for (int a = 0; a < NG; ++a) acc[r][c][a] = (R)0;
+                for (int a = 0; a < NG; ++a) {
+                    acc[r][c][a] = (R)0;
+                    if constexpr (C::BOTH) lost[r][c][a] = (R)0;
+                }
         for (int sl = 0; sl < SLOTS; ++sl) {
             const R* kp = Ke + (e0 + le) * (N * N);
             bool by_rows = false, on = true;
@@ -124,17 +128,8 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
             }
             if (!on) continue;
             const R* xp = sx + (sl * EB + le) * (N * NGP);
-            R part[C::NEST ? RPT : 1][C::NEST ? SC : 1][C::NEST ? NG : 1];
-            if constexpr (C::NEST) {
-#pragma unroll
-                for (int r = 0; r < RPT; ++r)
-#pragma unroll
-                    for (int c = 0; c < SC; ++c)
-#pragma unroll
-                        for (int a = 0; a < NG; ++a) part[r][c][a] = (R)0;
-            }
 #pragma unroll 1
-            for (int jc = 0; jc < N; jc += C::CH) {
+            for (int jc = 0; jc < N; jc += C::BL) {
                 R sum[RPT][SC][NG];   // short sums first: rounding grows with the square root of a chain's length
 #pragma unroll
                 for (int r = 0; r < RPT; ++r)
@@ -142,8 +137,25 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                     for (int c = 0; c < SC; ++c)
 #pragma unroll
                         for (int a = 0; a < NG; ++a) sum[r][c][a] = (R)0;
+                auto join = [&]() {
+#pragma unroll
+                    for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                        for (int c = 0; c < SC; ++c)
+#pragma unroll
+                            for (int a = 0; a < NG; ++a) {
+                                if constexpr (C::BOTH) {
+                                    const R add = sum[r][c][a] - lost[r][c][a], t = acc[r][c][a] + add;
+                                    lost[r][c][a] = (t - acc[r][c][a]) - add;
+                                    acc[r][c][a] = t;
+                                } else {
+                                    acc[r][c][a] += sum[r][c][a];
+                                }
+                                sum[r][c][a] = (R)0;
+                            }
+                };
 #pragma unroll 3
-                for (int j = jc; j < jc + C::CH; j += VJ) {
+                for (int j = jc; j < jc + C::BL; j += VJ) {
                     R kv[VJ][RPT];
                     if constexpr (C::BOTH) {
 #pragma unroll
@@ -158,7 +170,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                         for (int q = 0; q < VJ; ++q) kv[q][0] = __ldg(kp + (j + q) * N + row);
                     }
 #pragma unroll
-                    for (int q = 0; q < VJ; ++q)
+                    for (int q = 0; q < VJ; ++q) {
 #pragma unroll
                         for (int c = 0; c < SC; ++c) {
                             R xv[NGP];
@@ -174,24 +186,11 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
 #pragma unroll
                                 for (int a = 0; a < NG; ++a) sum[r][c][a] = fma(kv[q][r], xv[a], sum[r][c][a]);
                         }
+                        if constexpr (C::CH < C::BL)
+                            if ((q + 1) % C::CH == 0) join();
+                    }
                 }
-#pragma unroll
-                for (int r = 0; r < RPT; ++r)
-#pragma unroll
-                    for (int c = 0; c < SC; ++c)
-#pragma unroll
-                        for (int a = 0; a < NG; ++a) {
-                            if constexpr (C::NEST) part[r][c][a] += sum[r][c][a];
-                            else acc[r][c][a] += sum[r][c][a];
-                        }
-            }
-            if constexpr (C::NEST) {
-#pragma unroll
-                for (int r = 0; r < RPT; ++r)
-#pragma unroll
-                    for (int c = 0; c < SC; ++c)
-#pragma unroll
-                        for (int a = 0; a < NG; ++a) acc[r][c][a] += part[r][c][a];
+                if constexpr (C::CH == C::BL) join();
             }
         }
         const R rj = OWN ? rhoJ[e0 + le] : (R)0;

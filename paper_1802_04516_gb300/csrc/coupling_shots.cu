@@ -26,6 +26,7 @@ struct CouplingShots {
     static constexpr int NP = 6, NG = 3, N = 12, NV = 36, NK = N * N;
     static constexpr int CPR = NV / 4;                        // 16-byte pieces of a row (9: an odd stride, no bank conflicts)
     static constexpr int ROWS = 32 * NV;
+    static constexpr int CH = 6;                              // columns summed before they join the total
     template <int SH> static constexpr int buf() { return ROWS + 32 / SH * NK; }
     template <int SH> static constexpr size_t warp_bytes() { return sizeof(float) * 4 * buf<SH>(); }
 };
@@ -33,6 +34,13 @@ struct CouplingShots {
 __device__ __forceinline__ void cs_cp16(float* dst, const float* src, bool on) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 16u : 0u)
                  : "memory");
+}
+
+// compensated sum (Kahan 1965): the error of a total of 48 products stays that of its short sums
+__device__ __forceinline__ void cs_join(float& acc, float& lost, float sum) {
+    const float add = sum - lost, t = acc + add;
+    lost = (t - acc) - add;
+    acc = t;
 }
 
 template <int SH, bool OWN>
@@ -114,11 +122,11 @@ __global__ void __launch_bounds__(128) coupling_shots_kernel(int64_t n_elem, con
     issue(cur, 0, 2);
     for (int64_t t = 0; t < n_items; ++t) {
         const Item far = fetch(t + 2);
-        float2 acc[N / 2][NG];
+        float2 acc[N / 2][NG], lost[N / 2][NG];                // totals, what their last join rounded away
 #pragma unroll
         for (int i = 0; i < N / 2; ++i)
 #pragma unroll
-            for (int a = 0; a < NG; ++a) acc[i][a] = make_float2(0.f, 0.f);
+            for (int a = 0; a < NG; ++a) acc[i][a] = lost[i][a] = make_float2(0.f, 0.f);
         float out[N][NG];
 #pragma unroll
         for (int sl = 0; sl < 4; ++sl) {
@@ -136,21 +144,28 @@ __global__ void __launch_bounds__(128) coupling_shots_kernel(int64_t n_elem, con
             if (sl < 3 || OWN) {   // rows of a missing neighbour are zero (zero-filled copies)
                 const float4* kp = reinterpret_cast<const float4*>(buf + C::ROWS + sub * NK);
 #pragma unroll
-                for (int j = 0; j < N; ++j) {
-                    float2 kk[N / 2];
+                for (int g = 0; g < N / 4; ++g)                // four rows at a time: short sums, few registers
 #pragma unroll
-                    for (int q = 0; q < N / 4; ++q) {
-                        const float4 f = kp[j * (N / 4) + q];
-                        kk[2 * q] = make_float2(f.x, f.y);
-                        kk[2 * q + 1] = make_float2(f.z, f.w);
+                    for (int j0 = 0; j0 < N; j0 += C::CH) {
+                        float2 sum[2][NG];
+#pragma unroll
+                        for (int j = j0; j < j0 + C::CH; ++j) {
+                            const float4 f = kp[j * (N / 4) + g];
+#pragma unroll
+                            for (int a = 0; a < NG; ++a) {
+                                const float xv = v[(j / NP * NG + a) * NP + j % NP];
+                                sum[0][a] = ffma2(make_float2(f.x, f.y), make_float2(xv, xv), j > j0 ? sum[0][a] : make_float2(0.f, 0.f));
+                                sum[1][a] = ffma2(make_float2(f.z, f.w), make_float2(xv, xv), j > j0 ? sum[1][a] : make_float2(0.f, 0.f));
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int a = 0; a < NG; ++a) {
+                                cs_join(acc[2 * g + i][a].x, lost[2 * g + i][a].x, sum[i][a].x);
+                                cs_join(acc[2 * g + i][a].y, lost[2 * g + i][a].y, sum[i][a].y);
+                            }
                     }
-#pragma unroll
-                    for (int a = 0; a < NG; ++a) {
-                        const float xv = v[(j / NP * NG + a) * NP + j % NP];
-#pragma unroll
-                        for (int i = 0; i < N / 2; ++i) acc[i][a] = ffma2(kk[i], make_float2(xv, xv), acc[i][a]);
-                    }
-                }
             }
             if (sl == 3) {
                 const float rj = OWN && cur.e >= 0 ? rhoJ[cur.e] : 0.f;
