@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                                                              const R* __restrict__ rhoJ, const RefTables* __restrict__ rtp,
                                                              const R* __restrict__ x, const int* __restrict__ xidx, int64_t ld,
                                                              const R* __restrict__ base, const int* __restrict__ bidx,
-                                                             int64_t bld, R* __restrict__ y, R scale, int nshots,
+                                                             int64_t bld, R* __restrict__ y, double scale, int nshots,
                                                              int64_t nvec) {
     using C = Coupling<R, DIM, NP, NG, SC>;
     constexpr int N = C::N, FACES = C::FACES, NV = C::NV, RPT = C::RPT, TPE = C::TPE, NGP = C::NGP, VJ = C::VJ;
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
         for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sM[t] = (R)rtp->Mref[t];
     for (int t = threadIdx.x; t < NG * NG; t += blockDim.x) {
         if (OWN) sT[t] = (R)rtp->T[t];
-        sS[t] = scale * (R)rtp->S[t];
+        sS[t] = (R)(scale * rtp->S[t]);   // rounded once: its error is common to all elements
     }
     const int le = threadIdx.x / TPE, row = threadIdx.x % TPE;
     const bool act = le < ne;
@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                     R o = OWN ? (R)0 : SC == 1 ? bs[OWN || SC > 1 ? 0 : r][a] : base[at + a * NP];
 #pragma unroll
                     for (int b = 0; b < NG; ++b) {
+                        if constexpr (C::BOTH) o = fma(sS[a * NG + b], -lost[r][c][b], o);
                         o = fma(sS[a * NG + b], acc[r][c][b], o);
                         if (OWN) o = fma(sT[a * NG + b], u[b], o);
                     }
@@ -246,7 +247,7 @@ static cudaError_t coupling_go(stdg_ctx* c, const R* Ke, const R* Kf, const R* r
     auto kern = coupling_apply_kernel<R, DIM, NP, NG, SC, OWN>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<(unsigned)((c->n_elem + EB - 1) / EB), (EB * C::TPE + 31) / 32 * 32, smem, c->stream>>>(
-        c->n_elem, EB, c->d_adj, Ke, Kf, rhoJ, c->d_rt, x, xidx, ld, base, bidx, bld, y, (R)scale, nshots, c->nvel);
+        c->n_elem, EB, c->d_adj, Ke, Kf, rhoJ, c->d_rt, x, xidx, ld, base, bidx, bld, y, scale, nshots, c->nvel);
     note_launch(c);
     return cudaGetLastError();
 }

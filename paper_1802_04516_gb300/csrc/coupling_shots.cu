@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(128) coupling_shots_kernel(int64_t n_elem, con
                                                              const float* __restrict__ rhoJ, const RefTables* __restrict__ rtp,
                                                              const float* __restrict__ x, const int* __restrict__ xidx, int64_t ld,
                                                              const float* __restrict__ base, const int* __restrict__ bidx,
-                                                             int64_t bld, float* __restrict__ y, float scale, int nshots,
+                                                             int64_t bld, float* __restrict__ y, double scale, int nshots,
                                                              int64_t nvec) {
     using C = CouplingShots;
     constexpr int NP = C::NP, NG = C::NG, N = C::N, NV = C::NV, NK = C::NK, CPR = C::CPR, EPW = 32 / SH, BUF = C::ROWS + EPW * NK;
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(128) coupling_shots_kernel(int64_t n_elem, con
     for (int a = 0; a < NG; ++a)
 #pragma unroll
         for (int b = 0; b < NG; ++b) {
-            Sm[a][b] = scale * (float)rtp->S[a * NG + b];
+            Sm[a][b] = (float)(scale * rtp->S[a * NG + b]);   // rounded once: its error is common to all elements
             Tm[a][b] = OWN ? (float)rtp->T[a * NG + b] : 0.f;
         }
     __syncthreads();
@@ -187,6 +187,7 @@ __global__ void __launch_bounds__(128) coupling_shots_kernel(int64_t n_elem, con
                         float o = OWN ? 0.f : v[(k * NG + a) * NP + nn];
 #pragma unroll
                         for (int b = 0; b < NG; ++b) {
+                            o = fmaf(Sm[a][b], -(i % 2 ? lost[i / 2][b].y : lost[i / 2][b].x), o);
                             o = fmaf(Sm[a][b], i % 2 ? acc[i / 2][b].y : acc[i / 2][b].x, o);
                             if (OWN) o = fmaf(Tm[a][b], m[b], o);
                         }
@@ -236,7 +237,7 @@ static cudaError_t go(stdg_ctx* c, const float* x, const int* xidx, int64_t ld, 
     // two blocks an SM are resident (21 KB a warp): several rounds of them even out the tail
     const int64_t blocks = std::min<int64_t>((grp + wpb - 1) / wpb, (int64_t)c->n_sm * 8);
     kern<<<(unsigned)blocks, 32 * wpb, smem, c->stream>>>(c->n_elem, c->d_adj, c->d_Ke32, c->d_Kf32, c->d_rhoJ32, c->d_rt, x, xidx,
-                                                         ld, base, bidx, bld, y, (float)scale, nshots, c->nvel);
+                                                         ld, base, bidx, bld, y, scale, nshots, c->nvel);
     note_launch(c);
     return cudaGetLastError();
 }
