@@ -18,7 +18,7 @@ namespace stdg {
 // p_gamma = 2: 642 us with the face and mass kernels, 406 us here; 40,000 at p = 2: 398 and 154 us).  K_ii and the r
 // side's K_lr^T are read by columns (consecutive across the threads), the l side's K_lr by pieces of
 // its rows; the two ways of loading differ between the elements of a warp, the products do not.
-// FP32: bound by L1 wavefronts, then by HBM.  A thread has two or four consecutive rows, so that one
+// FP32: bound by L1 wavefronts, then by HBM.  A thread has two consecutive rows, so that one
 // 16-byte read of the staged values feeds them all, and the faces' blocks are kept in both
 // orientations, so that every load is a vector load of consecutive columns (reading rows of one copy
 // cost a wavefront per lane: 320 instead of 264 us on 200,704 triangles at p = 3).
