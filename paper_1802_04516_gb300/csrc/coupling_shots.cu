@@ -131,8 +131,12 @@ __global__ void __launch_bounds__(128) coupling_shots_kernel(int64_t n_elem, con
         float out[N][NG];
 #pragma unroll
         for (int sl = 0; sl < 4; ++sl) {
-            if (sl == 0) issue(cur, t, 3);
-            else issue(nxt, t + 1, sl - 1);
+            if (sl == 0) {
+                issue(cur, t, 3);                              // free since the end of the item before
+            } else {
+                __syncwarp();                                  // every lane has read the slot before: its buffer is free
+                issue(nxt, t + 1, sl - 1);
+            }
             asm volatile("cp.async.wait_group 3;" ::: "memory");
             __syncwarp();
             const float* buf = ring + sl * BUF;

@@ -105,3 +105,39 @@ def test_face_kernels_when_the_couplings_do_not_fit(p, pre):
         torch.cuda.empty_cache()
     assert held2 < held
     assert rel_l2(y2, y) < 1e-12 and rel_l2(z2, z) < 1e-10
+
+
+@pytest.mark.parametrize("shots", [25, 32, 57, 64, 90])
+@pytest.mark.parametrize("pre", [1, 2])
+def test_ring_of_slots_of_one_element_a_warp(shots, pre):
+    # 32 lanes on one element: its slot buffers are refilled by lanes other than their readers, across one to three
+    # chunks of shots. The off-diagonal form (stencil preconditioner) against the oracle; the form with the element's own
+    # block through one mixed slab, every shot against the same shot alone (rel_tol 1e-11, bar 1e-8 as for mixed states).
+    torch = need_gpu()
+    from oracle.precond import pre2
+    w = _workload(2, 2, 2, n=3)
+    s = _solver(w, precision="mixed", preconditioner=pre, rel_tol=1e-11, max_iters=20000)
+    s.set_shots(shots)
+    rng = np.random.default_rng(shots)
+    if pre == 2:
+        sim = oracle_sim(w)
+        P = pre2(sim.A, w.n_elem, sim.mesh.elem_nbr)
+        r = rng.normal(size=(shots, sim.A.shape[0]))
+        rd = torch.tensor(r, dtype=torch.float32, device="cuda")
+        zd = torch.zeros_like(rd)
+        torch.cuda.synchronize()
+        s.apply_preconditioner_device(w.dt, rd.data_ptr(), zd.data_ptr(), fp32=True)
+        z = zd.double().cpu().numpy()
+        for k in range(shots):
+            assert rel_l2(z[k], P @ r[k]) < 2e-3    # TF32 blocks
+    alone = _solver(w, precision="mixed", preconditioner=pre, rel_tol=1e-11, max_iters=20000)
+    alone.set_shots(1)
+    v0, sig0 = alone.get_state()
+    states = [(rng.normal(size=v0.shape), rng.normal(size=sig0.shape)) for _ in range(shots)]
+    for k, (v, sig) in enumerate(states):
+        s.set_state(v, sig, shot=k)
+    s.step(w.dt, 1)
+    for k in sorted({0, 7, 24, shots // 2, shots - 1}):
+        alone.set_state(*states[k])
+        alone.step(w.dt, 1)
+        assert rel_l2(s.get_state(k)[0], alone.get_state()[0]) < 1e-8
