@@ -728,9 +728,12 @@ __global__ void __launch_bounds__(kFinThreads) gm_cycle_end_kernel(DevScalars* s
     for (int s = threadIdx.x; s < ns; s += blockDim.x) any |= !ss[s].converged;
     any = __syncthreads_or(any);
     if (threadIdx.x == 0) {
+        // a cycle without an Arnoldi step (every unconverged shot has a NaN or Inf residual) left x as it
+        // was: the next one could do no better
+        const int go = any && sc->j > 0 && sc->iters < sc->max_iters;
         sc->j = 0;
         sc->runs[kBodyCycle] += 1;
-        sc->flag_outer = any && sc->iters < sc->max_iters;
+        sc->flag_outer = go;
         set_cond(h, use_h, sc->flag_outer);
     }
 }

@@ -176,3 +176,39 @@ def test_energy_sentinel_is_skipped_when_sources_drive_the_solution():
     s = gpu_solver(w, precision="fp64", rel_tol=1e-12, max_iters=5000)
     s.set_energy_check(True, -0.5)           # would trip on any source-free step
     assert s.step(w.dt, 2)["status"] == 0
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("pre", [0, 1, 2])
+@pytest.mark.parametrize("shots", [1, 3])
+def test_non_finite_residual_of_a_finite_right_hand_side_ends_the_restarts(precision, pre, shots):
+    # a finite state whose right-hand side has a finite norm but whose first residual overflows: no Arnoldi step can
+    # run, so the restart loop has to end by itself; stacked shots beside it converge as they do alone
+    need_gpu()
+    from paper_1802_04516_gb300.binding import STDG_ENONFINITE, Solver, StdgError
+    xyz, ev, per = synth.tri_grid(3, 2, 1.0, 1.0, periodic=False, jitter=0.2, seed=4)
+    rng = np.random.default_rng(3)
+    dt, bad = 2.0, shots // 2
+
+    def solver(n):
+        s = Solver(2, 2, 1, precision=precision, rel_tol=1e-10, max_iters=3000, gmres_restart=64, preconditioner=pre)
+        s.set_mesh(xyz, ev, per)
+        s.set_material(*synth.homogeneous(ev.shape[0], 2.0, 1.0, 1.0))
+        s.set_shots(n)
+        return s
+
+    s = solver(shots)
+    v0, sig0 = s.get_state(0)
+    states = [(rng.normal(size=v0.shape), rng.normal(size=sig0.shape)) for _ in range(shots)]
+    states[bad] = (1e153 * states[bad][0], 0 * sig0)
+    for k, st in enumerate(states):
+        s.set_state(*st, shot=k)
+    with pytest.raises(StdgError) as ei:
+        s.step(dt, 1)
+    assert ei.value.code == STDG_ENONFINITE and s.last_stats["iters_max"] < 3000
+    for k in range(shots):
+        if k != bad:
+            alone = solver(1)
+            alone.set_state(*states[k])
+            alone.step(dt, 1)
+            assert rel_l2(s.get_state(k)[0], alone.get_state()[0]) < 1e-7
