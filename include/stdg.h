@@ -296,7 +296,9 @@ int stdg_apply_preconditioner_device(stdg_ctx* ctx, double dt, const void* r_dev
  * A x is written into r_dev while x_dev is still being read.  The device address of the
  * array is looked up once per device and kept for the life of the process, so it assumes
  * the device's primary context is not reset (cudaDeviceReset) in between.  Asynchronous
- * on the context stream. */
+ * on the context stream.  A graph that a caller records from this call (or from the FP64
+ * stdg_apply_operator_device) reads the context's mesh and material arrays when it is
+ * replayed: it stays valid until the next stdg_set_mesh or stdg_destroy. */
 int stdg_residual_noalloc(stdg_ctx* ctx, double dt, const double* x_dev, const double* b_dev,
                           double* r_dev, double* out_dev);
 

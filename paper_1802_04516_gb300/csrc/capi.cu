@@ -929,7 +929,7 @@ int stdg_apply_operator_device(stdg_ctx* c, double dt, const void* x_dev, void* 
         STDG_CUDA(c, launch_apply32(c, dt, (const float*)x_dev, (float*)y_dev, 1.0));
         return take_device_error(c);   // the FP32 face kernel's bounded waits
     } else {
-        STDG_CUDA(c, launch_apply(c, dt, (const double*)x_dev, (double*)y_dev, 1.0));
+        STDG_CUDA(c, launch_apply_caller(c, dt, (const double*)x_dev, (double*)y_dev));
     }
     return STDG_OK;
 }

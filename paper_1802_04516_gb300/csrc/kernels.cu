@@ -786,12 +786,24 @@ static cudaError_t apply_tmpl(stdg_ctx* c, const R* D, const R* lamf, const R* m
 
 static double schur_c(const stdg_ctx* c) { return c->opt.scheme == STDG_SCHEME_CN ? 0.25 : 1.0; }
 
+// the operator from the face blocks, FP64
+static cudaError_t apply_faces(stdg_ctx* c, const double* x, double* y, double scale, const int* xidx, int64_t ld, int nshots) {
+    STDG_DISPATCH(c->dim, c->Nphi, return (apply_tmpl<D_, N_, double>(c, c->d_D, c->d_lamf, c->d_muf, c->d_rhoJ, x, y, scale, true, true, xidx, ld, nshots)));
+    return cudaSuccess;
+}
+
 cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, double cfac, const int* xidx, int64_t ld,
                          int nshots) {
     const double scale = cfac * schur_c(c) * dt * dt;
     if (c->d_Kf) return launch_coupling(c, x, xidx, ld, nullptr, nullptr, 0, y, scale, nshots);
-    STDG_DISPATCH(c->dim, c->Nphi, return (apply_tmpl<D_, N_, double>(c, c->d_D, c->d_lamf, c->d_muf, c->d_rhoJ, x, y, scale, true, true, xidx, ld, nshots)));
-    return cudaSuccess;
+    return apply_faces(c, x, y, scale, xidx, ld, nshots);
+}
+
+cudaError_t launch_apply_caller(stdg_ctx* c, double dt, const double* x, double* y) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    if (st == cudaStreamCaptureStatusNone) return launch_apply(c, dt, x, y, 1.0);
+    return apply_faces(c, x, y, schur_c(c) * dt * dt, nullptr, 0, 1);
 }
 
 // FP32: couplings or face kernels.  The two shapes with a tiled single-shot face kernel keep it, and

@@ -128,7 +128,7 @@ extern "C" int stdg_residual_noalloc(stdg_ctx* c, double dt, const double* x_dev
     double* parts = nullptr;
     int rc = scratch_address(c, &parts);
     if (rc != STDG_OK) return rc;
-    STDG_CUDA(c, launch_apply(c, dt, x_dev, r_dev, 1.0));
+    STDG_CUDA(c, launch_apply_caller(c, dt, x_dev, r_dev));
     const int nparts = (int)((n + kChunk - 1) / kChunk);
     residual_parts_kernel<<<nparts, kThreads, 0, c->stream>>>(n, b_dev, r_dev, parts);
     residual_total_kernel<<<1, kThreads, 0, c->stream>>>(nparts, parts, out_dev);

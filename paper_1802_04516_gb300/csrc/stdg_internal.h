@@ -228,6 +228,10 @@ cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, dou
                          const int* xidx = nullptr, int64_t ld = 0, int nshots = 1);
 cudaError_t launch_apply32(stdg_ctx* c, double dt, const float* x, float* y, double cfac,
                            const int* xidx = nullptr, int64_t ld = 0, int nshots = 1);
+// y = A x (FP64, one shot) on the stream for a caller of the library.  While the caller records that stream
+// into a graph of its own the operator runs from the face blocks, which stay where they are until the next
+// mesh: the graph outlives this call, and the couplings may be given back before it is replayed
+cudaError_t launch_apply_caller(stdg_ctx* c, double dt, const double* x, double* y);
 // w = A y for y = P_1 base (the exact block-Jacobi inverse, so D y = base): base plus the off-diagonal
 // couplings of y where the assembled couplings are kept, one ordinary application otherwise
 cudaError_t launch_apply_pre1(stdg_ctx* c, double dt, const double* y, const double* base, const int* bidx, int64_t bld,

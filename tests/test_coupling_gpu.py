@@ -141,3 +141,41 @@ def test_ring_of_slots_of_one_element_a_warp(shots, pre):
         alone.set_state(*states[k])
         alone.step(w.dt, 1)
         assert rel_l2(s.get_state(k)[0], alone.get_state()[0]) < 1e-8
+
+
+def test_recorded_operator_outlives_the_couplings():
+    # a caller's graph of the operator and of the residual, replayed after the couplings were given back (an allocation
+    # of the context that cannot succeed takes them first) and their room was overwritten
+    torch = need_gpu()
+    from paper_1802_04516_gb300 import binding
+    w = _workload(2, 2, 2, n=16)
+    stream = torch.cuda.Stream()
+    s = _solver(w, preconditioner=0, stream=stream.cuda_stream)
+    lib = binding.load()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x, b = (torch.randn(s.nvel, dtype=torch.float64, device="cuda", generator=g) for _ in range(2))
+    y, r, out = torch.zeros_like(x), torch.zeros_like(x), torch.zeros(2, dtype=torch.float64, device="cuda")
+
+    def calls():
+        s.apply_operator_device(w.dt, x.data_ptr(), y.data_ptr())
+        assert lib.stdg_residual_noalloc(s.h, w.dt, x.data_ptr(), b.data_ptr(), r.data_ptr(), out.data_ptr()) == 0
+
+    torch.cuda.synchronize()
+    calls()
+    torch.cuda.synchronize()
+    want = y.clone(), r.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        calls()
+    held = s.query(10)
+    with pytest.raises(binding.StdgError):
+        s.set_shots(1 << 24)
+    assert s.query(10) < held
+    junk = torch.full((1 << 27,), float("nan"), dtype=torch.float64, device="cuda")
+    y.fill_(float("nan"))
+    r.fill_(float("nan"))
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert rel_l2(y.cpu().numpy(), want[0].cpu().numpy()) < 1e-12 and rel_l2(r.cpu().numpy(), want[1].cpu().numpy()) < 1e-12
+    del junk
