@@ -113,9 +113,9 @@ int stdg_set_mesh(stdg_ctx* ctx, int64_t n_vert, const double* xyz, int64_t n_el
  * of its two elements.  Requires lambda >= 0, mu > 0, rho > 0, all finite (else
  * STDG_EINVAL); STDG_ESTATE before stdg_set_mesh.  Also sets up the preconditioner. */
 /* The operator's element couplings are laid out on the device with the medium, (d N_phi)^2 FP64
- * values per face and per element plus FP32 copies in mixed precision, where they take no more than a third of the free
- * memory; they are given back when a later allocation of the context needs the room, and the
- * operator then runs from the face blocks. */
+ * values per face and per element plus FP32 copies in mixed precision, where they take no more than
+ * their share of the free memory (stdg_set_coupling_share); they are given back when a later
+ * allocation of the context needs the room, and the operator then runs from the face blocks. */
 int stdg_set_material(stdg_ctx* ctx, const double* lambda, const double* mu, const double* rho);
 
 /* Per-element time scale alpha (n_elem values, > 0, finite), for disconnected parts of one
@@ -216,7 +216,8 @@ int stdg_apply_operator_device(stdg_ctx* ctx, double dt, const void* x_dev, void
  * 10 device bytes held, 11 kernel executions of the library during the last stdg_step
  * call (counted on the device, including every iteration of the device-side loops),
  * 12 bits per stored entry of the stencil preconditioner's local blocks in the FP32 inner
- * solve of one shot (16 or 32; 0 without such blocks). */
+ * solve of one shot (16 or 32; 0 without such blocks), 13 device bytes of the operator's element
+ * couplings (0 while the operator runs from the face blocks). */
 int stdg_query(stdg_ctx* ctx, int what, int64_t* out);
 
 /* Storage of the stencil preconditioner's local blocks S_e^{-1} (Appendix A, Eq. APPRE2)
@@ -228,6 +229,13 @@ int stdg_query(stdg_ctx* ctx, int what, int64_t* out);
  * iteration, so the solution meets the same residual bar either way.  Shapes with an odd
  * d N_phi N_gamma or above 128 keep FP32.  Returns STDG_OK or STDG_EINVAL (bits not 16/32). */
 int stdg_set_pre2_storage(stdg_ctx* ctx, int bits);
+
+/* Most of the device's free memory, 0 <= share <= 1 (default 1/16), that the operator's element
+ * couplings may take when stdg_set_material or stdg_set_time_scale lays them out; what they leave
+ * is there for other contexts, libraries and processes on the device, whose allocations cannot take
+ * it back.  0 gives couplings that are held back at once and runs the operator from the face blocks.
+ * Returns STDG_OK or STDG_EINVAL. */
+int stdg_set_coupling_share(stdg_ctx* ctx, double share);
 
 /* Face table as built by stdg_set_mesh: l(j), r(j) (-1 on the boundary). */
 int stdg_get_faces(stdg_ctx* ctx, int32_t* face_l, int32_t* face_r);

@@ -67,6 +67,7 @@ SIGNATURES = {
     "stdg_set_energy_check": (C.c_int, [_P, C.c_int, C.c_double]),
     "stdg_set_time_scale": (C.c_int, [_P, _D]),
     "stdg_set_pre2_storage": (C.c_int, [_P, C.c_int]),
+    "stdg_set_coupling_share": (C.c_int, [_P, C.c_double]),
     "stdg_read_receivers": (C.c_int, [_P, _D, C.c_int64]),
     "stdg_apply_operator": (C.c_int, [_P, C.c_double, _D, _D]),
     "stdg_apply_operator_device": (C.c_int, [_P, C.c_double, _P, _P, C.c_int]),
@@ -325,6 +326,13 @@ class Solver:
         self._chk(self.lib.stdg_set_pre2_storage(self.h, int(bits)))
 
     pre2_bits = property(lambda s: s.query(12))
+
+    def set_coupling_share(self, share):
+        """Most of the device's free memory that the operator's element couplings may take when the material is
+        set (default 1/16); 0 gives them back at once and runs the operator from the face blocks."""
+        self._chk(self.lib.stdg_set_coupling_share(self.h, float(share)))
+
+    coupling_bytes = property(lambda s: s.query(13))
 
     def set_energy_check(self, enable=True, rel_tol=0.0):
         """Energy-growth sentinel around step (Theorem 4): STDG_EENERGY when a shot's energy

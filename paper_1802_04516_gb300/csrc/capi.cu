@@ -165,15 +165,16 @@ static int ensure_fp32(stdg_ctx* c) {
     return STDG_OK;
 }
 
-// Assembled couplings of the current medium (FP64, and their FP32 copy where D~ has one).  They are
-// left out where they would take more than a third of the free memory.
+// Assembled couplings of the current medium (FP64, and their FP32 copy where D~ has one), where they
+// fit the share of the free memory that they may take.  Only this context can take their room back, so
+// the default share is small: the largest benchmark mesh (200,704 triangles, p = 3) needs 1.6 of 280 GB.
 static int setup_coupling(stdg_ctx* c) {
     const int64_t n2 = (int64_t)c->dim * c->Nphi * c->dim * c->Nphi, nKf = c->n_face * n2, nKe = c->n_elem * n2;
     const bool want32 = c->d_D32 != nullptr && coupling32_wanted(c);
     if (!c->d_Kf) {
         size_t free_b = 0, total_b = 0;
         STDG_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
-        if ((size_t)(nKf + nKe) * (want32 ? 16 : 8) > free_b / 3) return STDG_OK;
+        if ((double)(nKf + nKe) * (want32 ? 16 : 8) > c->coupling_share * (double)free_b) return STDG_OK;
         double *kf = nullptr, *ke = nullptr;
         if (dev_alloc(c, (void**)&kf, sizeof(double) * nKf) != STDG_OK || dev_alloc(c, (void**)&ke, sizeof(double) * nKe) != STDG_OK) {
             dev_release(c, kf);
@@ -951,6 +952,11 @@ int stdg_query(stdg_ctx* c, int what, int64_t* out) {
         case 10: *out = (int64_t)c->bytes; break;
         case 11: *out = c->last_launches; break;
         case 12: *out = c->d_pre2_32 ? (c->d_pre2_16 && c->pre2_bits == 16 ? 16 : 32) : 0; break;
+        case 13: {
+            const int64_t n2 = (int64_t)c->dim * c->Nphi * c->dim * c->Nphi;
+            *out = (c->d_Kf ? 8 * n2 * (c->n_face + c->n_elem) : 0) + (c->d_Kf32 ? 4 * n2 * (2 * c->n_face + c->n_elem) : 0);
+            break;
+        }
         default: STDG_FAIL(c, STDG_EINVAL, "unknown query");
     }
     return STDG_OK;
@@ -961,6 +967,14 @@ int stdg_set_pre2_storage(stdg_ctx* c, int bits) {
     if (bits != 16 && bits != 32) STDG_FAIL(c, STDG_EINVAL, "bits must be 16 or 32");
     c->pre2_bits = bits;
     solver_invalidate_graph(c);   // graphs keep the kernel they were captured with
+    return STDG_OK;
+}
+
+int stdg_set_coupling_share(stdg_ctx* c, double share) {
+    CHECK_CTX(c);
+    if (!(share >= 0.0 && share <= 1.0)) STDG_FAIL(c, STDG_EINVAL, "share must be between 0 and 1");
+    c->coupling_share = share;
+    if (share == 0.0 && c->d_Kf) drop_coupling(c);
     return STDG_OK;
 }
 

@@ -179,3 +179,62 @@ def test_recorded_operator_outlives_the_couplings():
     torch.cuda.synchronize()
     assert rel_l2(y.cpu().numpy(), want[0].cpu().numpy()) < 1e-12 and rel_l2(r.cpu().numpy(), want[1].cpu().numpy()) < 1e-12
     del junk
+
+
+@pytest.mark.parametrize("room,share,held", [(6, None, False), (30, None, True), (6, 0.5, True), (30, 0.0, False)])
+def test_couplings_take_no_more_than_their_share_of_the_free_memory(room, share, held):
+    # a mesh whose couplings are 1/room of the memory that is free when they are laid out (the rest stays for others):
+    # by default they may take 1/16 of it
+    torch = need_gpu()
+    w = _workload(2, 3, 3, n=120)
+    x = np.random.default_rng(8).normal(size=w.n_elem * 80)
+
+    def run(share):
+        from paper_1802_04516_gb300.binding import Solver
+        s = Solver(2, 3, 3, preconditioner=0)
+        try:
+            if share is not None:
+                s.set_coupling_share(share)
+            s.set_mesh(w.xyz, w.elem_vert, w.period)
+            s.set_material(w.lam, w.mu, w.rho)
+            return s.apply_operator(w.dt, x), s.query(10), s.coupling_bytes
+        finally:
+            s.close()
+
+    y0, base, none = run(0.0)
+    assert none == 0
+    y1, full, couplings = run(1.0)
+    assert couplings == full - base > 0
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    fill = torch.empty(free - base - room * couplings, dtype=torch.uint8, device="cuda")
+    try:
+        y, _, c = run(share)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert (c > 0) == held
+    assert rel_l2(y, y0) < 1e-12 and rel_l2(y1, y0) < 1e-12
+
+
+def test_couplings_given_back_at_once():
+    need_gpu()
+    from paper_1802_04516_gb300.binding import STDG_EINVAL, StdgError
+    w = _workload(2, 2, 2, n=4)
+    s = _solver(w, precision="mixed", preconditioner=2)
+    x = np.random.default_rng(8).normal(size=s.nvel)
+    y = s.apply_operator(w.dt, x)
+    held, c = s.query(10), s.coupling_bytes
+    assert c > 0
+    for bad in (-0.1, 1.5, float("nan")):
+        with pytest.raises(StdgError) as ei:
+            s.set_coupling_share(bad)
+        assert ei.value.code == STDG_EINVAL
+    s.set_coupling_share(0.0)
+    assert s.coupling_bytes == 0 and s.query(10) == held - c
+    assert rel_l2(s.apply_operator(w.dt, x), y) < 1e-12
+    s.set_material(w.lam, w.mu, w.rho)
+    assert s.coupling_bytes == 0
+    s.set_coupling_share(1.0)
+    s.set_material(w.lam, w.mu, w.rho)
+    assert s.coupling_bytes == c
