@@ -439,8 +439,6 @@ static cudaError_t go(stdg_ctx* c, double dt, const R* Ke, const R* Kf, const R*
     constexpr int N = DIM * NP;
     if (const int epc = cluster_elements(c)) {
         auto kern = cg_cluster_kernel<R, DIM, NP>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
         cudaLaunchAttribute at{};
         at.id = cudaLaunchAttributeClusterDimension;
         at.val.clusterDim.x = kClusterSize;
@@ -451,9 +449,16 @@ static cudaError_t go(stdg_ctx* c, double dt, const R* Ke, const R* Kf, const R*
         cfg.stream = c->stream;
         cfg.attrs = &at;
         cfg.numAttrs = 1;
-        note_launch(c);
-        return cudaLaunchKernelEx(&cfg, kern, c->n_elem, epc, (const int2*)c->d_adj, Ke, Kf, rhoJ, (const RefTables*)c->d_rt,
-                                  (R)(0.25 * dt * dt), V, B, x, r, z, p, sc, ss, h, use_h);
+        // 16 blocks are more than the portable cluster size: a partition of the GPU, or one whose clusters hold
+        // fewer free SMs, cannot schedule them, and the two kernels below serve every size
+        int fit = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit > 0) {
+            note_launch(c);
+            return cudaLaunchKernelEx(&cfg, kern, c->n_elem, epc, (const int2*)c->d_adj, Ke, Kf, rhoJ, (const RefTables*)c->d_rt,
+                                      (R)(0.25 * dt * dt), V, B, x, r, z, p, sc, ss, h, use_h);
+        }
+        cudaGetLastError();
     }
     // whole warps of rows, at most 160 threads; at least one block per SM on small meshes, and on large
     // ones at most four, so that the reductions stay short

@@ -2,11 +2,16 @@
 than one block, shots whose segments start off a 16-byte boundary, restart lengths around the 16
 columns that one pass of the multi-dot kernel takes, and shots that converge at different steps.
 Every shot against its own oracle run, at the stated state bars (1e-10 FP64, 1e-8 mixed)."""
+import os
+import shutil
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 import synth
-from helpers import need_gpu, oracle_sim, rel_l2
+from helpers import ROOT, need_gpu, oracle_sim, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +103,62 @@ def test_crank_nicolson_around_the_cluster_limit(nx, ny, p, precision):
     s.step(w.dt, 2)
     out, _ = s.get_state()
     assert rel_l2(out, sim.v_tr) < (1e-10 if precision == "fp64" else 1e-8)
+
+
+# runtime of a device that cannot schedule a cluster of 16 blocks: the occupancy query answers none, a launch fails
+NO_CLUSTERS = r"""
+#include <dlfcn.h>
+#include <cuda_runtime_api.h>
+extern "C" cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) {
+    *n = 0;
+    return cudaSuccess;
+}
+extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* cfg, const void* f, void** args) {
+    for (unsigned i = 0; i < cfg->numAttrs; ++i)
+        if (cfg->attrs[i].id == cudaLaunchAttributeClusterDimension && cfg->attrs[i].val.clusterDim.x > 8)
+            return cudaErrorInvalidClusterSize;
+    using F = cudaError_t (*)(const cudaLaunchConfig_t*, const void*, void**);
+    return ((F)dlsym(RTLD_NEXT, "cudaLaunchKernelExC"))(cfg, f, args);
+}
+"""
+
+SMALL_CN = """
+import sys
+import numpy as np
+sys.path.insert(0, {root!r})
+import synth
+from paper_1802_04516_gb300.binding import Solver
+xyz, ev, per = synth.tri_grid(8, 7, 1.0, 1.0, periodic=False, jitter=0.2, seed=6)
+out = []
+for precision, use_graph in (("fp64", True), ("mixed", True), ("fp64", False)):
+    s = Solver(2, 2, 0, scheme="cn", precision=precision, rel_tol=1e-13 if precision == "fp64" else 1e-12, max_iters=20000,
+               preconditioner=1, use_graph=use_graph)
+    s.set_mesh(xyz, ev, per)
+    s.set_material(*synth.homogeneous(ev.shape[0], 2.0, 1.0, 1.0))
+    v, sig = s.get_state()
+    rng = np.random.default_rng(12)
+    s.set_state(rng.normal(size=v.shape), rng.normal(size=sig.shape))
+    s.step(0.02, 2)
+    out.append(s.get_state()[0])
+np.save(sys.argv[1], np.array(out))
+"""
+
+
+def test_small_crank_nicolson_without_clusters_of_sixteen(tmp_path):
+    need_gpu()
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no C++ compiler")
+    src, lib = tmp_path / "fake.cpp", tmp_path / "fake.so"
+    src.write_text(NO_CLUSTERS)
+    subprocess.run([gxx, "-shared", "-fPIC", "-I", "/usr/local/cuda/include", "-o", str(lib), str(src), "-ldl"], check=True)
+    got = []
+    for fake in (False, True):
+        env = dict(os.environ, LD_PRELOAD=str(lib)) if fake else dict(os.environ)
+        path = tmp_path / ("%d.npy" % fake)
+        r = subprocess.run([sys.executable, "-c", SMALL_CN.format(root=ROOT), str(path)], env=env, capture_output=True, text=True)
+        assert r.returncode == 0, r.stderr
+        got.append(np.load(path))
+    for k, tol in enumerate((1e-10, 1e-8, 1e-10)):
+        assert rel_l2(got[1][k], got[0][k]) < tol
+    assert not np.array_equal(got[1][0], got[0][0])   # the runtime was the fake one: another order of the sums
