@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "compensated.h"
 #include "stdg_internal.h"
 
 namespace stdg {
@@ -31,7 +32,7 @@ struct Coupling {
     static constexpr int NGP = NG <= 2 ? NG : (NG <= 4 ? 4 : 6);          // row stride of the staged values
     static constexpr int VJ = !BOTH || SC > 1 ? 2 : (N % 10 == 0 ? 10 : 6);   // columns loaded together
     static constexpr int BL = !BOTH ? N : (N % 10 == 0 ? 10 : 6);         // columns per turn of the loop
-    // FP32: columns summed before they join the total, and the joins are compensated (Kahan 1965)
+    // FP32: columns summed before they join the total (compensated.h)
     static constexpr int CH = !BOTH || SC > 1 ? BL : BL / 2;
     static_assert(N % BL == 0 && BL % VJ == 0 && (CH == BL || (VJ == BL && VJ % CH == 0)), "chunks of whole loads");
     static_assert(N % 2 == 0, "d N_phi is even for every supported order");
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                 for (int a = 0; a < NG; ++a) bs[r][a] = base[(int64_t)s0 * nvec + (e0 + le) * NV + (k * NG + a) * NP + nn];
             }
         }
-        R acc[RPT][SC][NG], lost[C::BOTH ? RPT : 1][C::BOTH ? SC : 1][C::BOTH ? NG : 1];   // totals, what their last join rounded away
+        R acc[RPT][SC][NG], low[C::BOTH ? RPT : 1][C::BOTH ? SC : 1][C::BOTH ? NG : 1];   // totals, what their joins rounded away
 #pragma unroll
         for (int r = 0; r < RPT; ++r)
 #pragma unroll
@@ -112,7 +113,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
 #pragma unroll
                 for (int a = 0; a < NG; ++a) {
                     acc[r][c][a] = (R)0;
-                    if constexpr (C::BOTH) lost[r][c][a] = (R)0;
+                    if constexpr (C::BOTH) low[r][c][a] = (R)0;
                 }
         for (int sl = 0; sl < SLOTS; ++sl) {
             const R* kp = Ke + (e0 + le) * (N * N);
@@ -137,20 +138,15 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                     for (int c = 0; c < SC; ++c)
 #pragma unroll
                         for (int a = 0; a < NG; ++a) sum[r][c][a] = (R)0;
-                auto join = [&]() {
+                auto join_all = [&]() {
 #pragma unroll
                     for (int r = 0; r < RPT; ++r)
 #pragma unroll
                         for (int c = 0; c < SC; ++c)
 #pragma unroll
                             for (int a = 0; a < NG; ++a) {
-                                if constexpr (C::BOTH) {
-                                    const R add = sum[r][c][a] - lost[r][c][a], t = acc[r][c][a] + add;
-                                    lost[r][c][a] = (t - acc[r][c][a]) - add;
-                                    acc[r][c][a] = t;
-                                } else {
-                                    acc[r][c][a] += sum[r][c][a];
-                                }
+                                if constexpr (C::BOTH) join(acc[r][c][a], low[r][c][a], sum[r][c][a]);
+                                else acc[r][c][a] += sum[r][c][a];
                                 sum[r][c][a] = (R)0;
                             }
                 };
@@ -187,10 +183,10 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                                 for (int a = 0; a < NG; ++a) sum[r][c][a] = fma(kv[q][r], xv[a], sum[r][c][a]);
                         }
                         if constexpr (C::CH < C::BL)
-                            if ((q + 1) % C::CH == 0) join();
+                            if ((q + 1) % C::CH == 0) join_all();
                     }
                 }
-                if constexpr (C::CH == C::BL) join();
+                if constexpr (C::CH == C::BL) join_all();
             }
         }
         const R rj = OWN ? rhoJ[e0 + le] : (R)0;
@@ -219,7 +215,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                     R o = OWN ? (R)0 : SC == 1 ? bs[OWN || SC > 1 ? 0 : r][a] : base[at + a * NP];
 #pragma unroll
                     for (int b = 0; b < NG; ++b) {
-                        if constexpr (C::BOTH) o = fma(sS[a * NG + b], -lost[r][c][b], o);
+                        if constexpr (C::BOTH) o = fma(sS[a * NG + b], rest(acc[r][c][b], low[r][c][b]), o);
                         o = fma(sS[a * NG + b], acc[r][c][b], o);
                         if (OWN) o = fma(sT[a * NG + b], u[b], o);
                     }

@@ -238,3 +238,24 @@ def test_couplings_given_back_at_once():
     s.set_coupling_share(1.0)
     s.set_material(w.lam, w.mu, w.rho)
     assert s.coupling_bytes == c
+
+
+@pytest.mark.parametrize("dim,p", [(2, 1), (2, 3), (3, 1)])
+def test_fp32_results_that_overflow_are_infinite(dim, p):
+    # one large value: every row is one product (plus the mass term), scaled by dt^2 / 4 at the end; results far above
+    # the largest FP32 number are infinite, those whose product before the scaling is far below it are finite
+    torch = need_gpu()
+    w = _workload(dim, p, 0)
+    w.lam[:], w.mu[:], w.scheme = w.lam * 1e12, w.mu * 1e12, "cn"
+    s = _solver(w, precision="mixed", preconditioner=0)
+    x = np.zeros(s.nvel)
+    x[s.nvel // 2] = 1e30
+    ref = s.apply_operator(w.dt, x)
+    xd = torch.tensor(x, dtype=torch.float32, device="cuda")
+    yd = torch.zeros_like(xd)
+    torch.cuda.synchronize()
+    s.apply_operator_device(w.dt, xd.data_ptr(), yd.data_ptr(), fp32=True)
+    y = yd.double().cpu().numpy()
+    big, small = np.abs(ref) > 1e39, np.abs(ref) < 1e38 * w.dt ** 2 / 4
+    assert big.any() and np.array_equal(y[big], np.sign(ref[big]) * np.inf)
+    assert np.isfinite(y[small]).all()
