@@ -20,6 +20,7 @@
 
 #include <cooperative_groups.h>
 
+#include "compensated.h"
 #include "krylov.h"
 #include "stdg_internal.h"
 
@@ -32,13 +33,13 @@ template <> struct CgPair<double> { using T = double2; };
 template <typename R, int DIM, int NP>
 __global__ void __launch_bounds__(160) cg_apply_kernel(int64_t n_elem, int EB, const int2* __restrict__ adj,
                                                        const R* __restrict__ Ke, const R* __restrict__ Kf,
-                                                       const R* __restrict__ rhoJ, const RefTables* __restrict__ rtp, R scale,
+                                                       const R* __restrict__ rhoJ, const RefTables* __restrict__ rtp, double scale,
                                                        const R* __restrict__ z, const R* p0, const R* p1, R* pw0, R* pw1,
                                                        R* __restrict__ q, const DevScalars* __restrict__ sc, ShotScalars* ss,
                                                        double* part, unsigned* done) {
     constexpr int N = DIM * NP, FACES = DIM + 1, SLOTS = FACES + 1;
     constexpr bool BOTH = sizeof(R) == 4;                     // the FP32 faces' blocks are kept in both orientations
-    constexpr int CH = N % 10 == 0 ? 10 : 6;                  // FP32 sums in short chains, as the stand-alone operator
+    constexpr int CH = N % 10 == 0 ? 10 : 6;                  // columns loaded together
     using P = typename CgPair<R>::T;
     extern __shared__ __align__(16) unsigned char smraw[];
     R* sx = reinterpret_cast<R*>(smraw);                      // [slot][element][row]
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(160) cg_apply_kernel(int64_t n_elem, int EB, c
     const double beta = ss->beta, rz = ss->pq;
     const R* po = odd ? p1 : p0;
     R* pn = odd ? pw0 : pw1;
-    const R S = scale * (R)rtp->S[0], T = (R)rtp->T[0];
+    const R S = (R)(scale * rtp->S[0]), T = (R)rtp->T[0];   // rounded once
     for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sM[t] = (R)rtp->Mref[t];
     const int le = threadIdx.x / N, row = threadIdx.x % N;
     Acc<R> pq;
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(160) cg_apply_kernel(int64_t n_elem, int EB, c
         }
         __syncthreads();
         if (!act) continue;
-        R acc = (R)0;
+        RowSum<R> acc;
 #pragma unroll
         for (int sl = 0; sl < SLOTS; ++sl) {
             const R* kp = Ke + e * (N * N);
@@ -89,7 +90,6 @@ __global__ void __launch_bounds__(160) cg_apply_kernel(int64_t n_elem, int EB, c
                 kp = Kf + (int64_t)(BOTH ? a.y : a.y >> 1) * (N * N);
             }
             const R* xp = sx + (sl * EB + le) * N;
-            R slot = (R)0;
             for (int jc = 0; jc < N; jc += CH) {
                 R kv[CH];
                 if (by_rows) {
@@ -103,18 +103,15 @@ __global__ void __launch_bounds__(160) cg_apply_kernel(int64_t n_elem, int EB, c
 #pragma unroll
                     for (int j = 0; j < CH; ++j) kv[j] = __ldg(kp + (jc + j) * N + row);
                 }
-                R sum = (R)0;
-#pragma unroll
-                for (int j = 0; j < CH; ++j) sum = fma(kv[j], xp[jc + j], sum);
-                slot += sum;
+                acc.columns(kv, [&](int j) { return xp[jc + j]; });
             }
-            acc += slot;
+            acc.end_slot();
         }
         const int k = row / NP, nn = row % NP;
         R u = (R)0;
 #pragma unroll
         for (int j = 0; j < NP; ++j) u = fma(sM[nn * NP + j], sx[le * N + k * NP + j], u);
-        const R o = fma(T, u * rhoJ[e], S * acc);
+        const R o = fma(T, u * rhoJ[e], acc.scaled(S));
         q[e * N + row] = o;
         pq.add(own, o);
     }
@@ -221,7 +218,7 @@ constexpr int kClusterSize = 16;
 template <typename R, int DIM, int NP>
 __global__ void __launch_bounds__(512, 1) cg_cluster_kernel(int64_t n_elem, int EPC, const int2* __restrict__ adj,
                                                             const R* __restrict__ Ke, const R* __restrict__ Kf,
-                                                            const R* __restrict__ rhoJ, const RefTables* __restrict__ rtp, R scale,
+                                                            const R* __restrict__ rhoJ, const RefTables* __restrict__ rtp, double scale,
                                                             const R* __restrict__ V, const R* __restrict__ B, R* x, R* r, R* z,
                                                             R* p, DevScalars* sc, ShotScalars* ss, cudaGraphConditionalHandle h,
                                                             int use_h) {
@@ -236,7 +233,7 @@ __global__ void __launch_bounds__(512, 1) cg_cluster_kernel(int64_t n_elem, int 
     __shared__ double part[3], bc[2];
     const int rank = blockIdx.x, CT = gridDim.x;
     for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sM[t] = (R)rtp->Mref[t];
-    const R S = scale * (R)rtp->S[0], T = (R)rtp->T[0];
+    const R S = (R)(scale * rtp->S[0]), T = (R)rtp->T[0];   // rounded once
     const int le = threadIdx.x / N, row = threadIdx.x % N, k = row / NP, nn = row % NP;
     const int64_t e = (int64_t)rank * EPC + le, at = e * N + row;
     const bool act = le < EPC && e < n_elem;
@@ -319,11 +316,10 @@ __global__ void __launch_bounds__(512, 1) cg_cluster_kernel(int64_t n_elem, int 
 #pragma unroll
                     for (int j = 0; j < N; ++j) pn[i][j] = nb[i].x >= 0 ? __ldcg(p + (int64_t)nb[i].x * N + j) : (R)0;
             }
-            R acc = (R)0;
+            RowSum<R> acc;
 #pragma unroll
             for (int sl = 0; sl < SLOTS; ++sl) {
                 if (sl && nb[sl ? sl - 1 : 0].x < 0) continue;
-                R slot = (R)0;
 #pragma unroll 1
                 for (int jc = 0; jc < N; jc += CH) {
                     R kv[CH];
@@ -333,23 +329,18 @@ __global__ void __launch_bounds__(512, 1) cg_cluster_kernel(int64_t n_elem, int 
                     } else {
                         load_k(sl, jc, kv);
                     }
-                    R sum = (R)0;
-#pragma unroll
-                    for (int j = 0; j < CH; ++j) {
-                        R pj;
-                        if (sl == 0) pj = sp[le * N + jc + j];
-                        else if constexpr (N <= 6) pj = pn[sl ? sl - 1 : 0][j];
-                        else pj = __ldcg(p + (int64_t)nb[sl ? sl - 1 : 0].x * N + jc + j);
-                        sum = fma(kv[j], pj, sum);
-                    }
-                    slot += sum;
+                    acc.columns(kv, [&](int j) {
+                        if (sl == 0) return sp[le * N + jc + j];
+                        if constexpr (N <= 6) return pn[sl ? sl - 1 : 0][j];
+                        else return __ldcg(p + (int64_t)nb[sl ? sl - 1 : 0].x * N + jc + j);
+                    });
                 }
-                acc += slot;
+                acc.end_slot();
             }
             R u = (R)0;
 #pragma unroll
             for (int j = 0; j < NP; ++j) u = fma(sM[nn * NP + j], sp[le * N + k * NP + j], u);
-            q = fma(T, u * rj, S * acc);
+            q = fma(T, u * rj, acc.scaled(S));
             pq.add(pv, q);
         }
         {
@@ -456,7 +447,7 @@ static cudaError_t go(stdg_ctx* c, double dt, const R* Ke, const R* Kf, const R*
             cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit > 0) {
             note_launch(c);
             return cudaLaunchKernelEx(&cfg, kern, c->n_elem, epc, (const int2*)c->d_adj, Ke, Kf, rhoJ, (const RefTables*)c->d_rt,
-                                      (R)(0.25 * dt * dt), V, B, x, r, z, p, sc, ss, h, use_h);
+                                      0.25 * dt * dt, V, B, x, r, z, p, sc, ss, h, use_h);
         }
         cudaGetLastError();
     }
@@ -472,7 +463,7 @@ static cudaError_t go(stdg_ctx* c, double dt, const R* Ke, const R* Kf, const R*
     const unsigned grid = (unsigned)std::min<int64_t>((c->n_elem + EB - 1) / EB, (int64_t)c->n_sm * 4);
     const int threads = (EB * N + 31) / 32 * 32;
     cg_apply_kernel<R, DIM, NP><<<grid, threads, sizeof(R) * (DIM + 2) * EB * N, c->stream>>>(
-        c->n_elem, EB, c->d_adj, Ke, Kf, rhoJ, c->d_rt, (R)(0.25 * dt * dt), z, p, pb, p, pb, q, sc, ss, part, done);
+        c->n_elem, EB, c->d_adj, Ke, Kf, rhoJ, c->d_rt, 0.25 * dt * dt, z, p, pb, p, pb, q, sc, ss, part, done);
     note_launch(c);
     cg_update_kernel_fused<R, DIM, NP><<<grid, threads, sizeof(R) * 2 * EB * N, c->stream>>>(
         c->n_elem, EB, V, B, x, r, z, p, pb, q, sc, ss, part, done, h, use_h);

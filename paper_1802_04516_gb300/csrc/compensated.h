@@ -5,6 +5,7 @@
 // infinite total stays infinite instead of turning into Inf - Inf).
 // Plain C++ for the host as well, so that the arithmetic can be tested without a GPU.
 #pragma once
+#include <cmath>
 
 #ifdef __CUDACC__
 #define STDG_HD __host__ __device__ __forceinline__
@@ -23,5 +24,35 @@ STDG_HD void join(float& total, float& low, float sum) {
 
 // the collected errors, to be added to the total last (none where the total is not finite)
 STDG_HD float rest(float total, float low) { return total - total == 0.f ? low : 0.f; }
+
+// Sum of a row's products over the couplings, CH columns at a time.  FP64: a chain per neighbour, then their
+// sum.  FP32: as the operator by itself (coupling_apply.h), chains of half as many columns joined with
+// compensation; plain totals had 4% (2D p = 1) to 7% (3D p = 1) more error than the face form's.
+template <typename R> struct RowSum;
+template <> struct RowSum<double> {
+    double total = 0.0, slot = 0.0;
+    template <int CH, class F> STDG_HD void columns(const double (&kv)[CH], F&& x) {
+        double sum = 0.0;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) sum = fma(kv[j], x(j), sum);
+        slot += sum;
+    }
+    STDG_HD void end_slot() { total += slot; slot = 0.0; }
+    STDG_HD double scaled(double S) const { return S * total; }
+};
+template <> struct RowSum<float> {
+    float total = 0.f, low = 0.f;
+    template <int CH, class F> STDG_HD void columns(const float (&kv)[CH], F&& x) {
+#pragma unroll
+        for (int c = 0; c < CH; c += CH / 2) {
+            float sum = 0.f;
+#pragma unroll
+            for (int j = c; j < c + CH / 2; ++j) sum = fmaf(kv[j], x(j), sum);
+            join(total, low, sum);
+        }
+    }
+    STDG_HD void end_slot() {}
+    STDG_HD float scaled(float S) const { return fmaf(S, total, S * rest(total, low)); }
+};
 
 }  // namespace stdg

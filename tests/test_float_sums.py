@@ -12,6 +12,21 @@ from helpers import ROOT
 
 SRC = r"""
 #include "compensated.h"
+template <int CH> static float row(const float* k, const float* x, int slots, int n) {
+    stdg::RowSum<float> r;
+    for (int s = 0; s < slots; ++s) {
+        for (int c = 0; c < n; c += CH) {
+            float kv[CH];
+            for (int j = 0; j < CH; ++j) kv[j] = k[s * n + c + j];
+            r.columns(kv, [&](int j) { return x[s * n + c + j]; });
+        }
+        r.end_slot();
+    }
+    return r.scaled(1.f);
+}
+extern "C" float row_sum(const float* k, const float* x, int slots, int n) {
+    return n % 10 == 0 ? row<10>(k, x, slots, n) : row<6>(k, x, slots, n);
+}
 extern "C" float joined(const float* x, int n) {
     float total = 0.f, low = 0.f;
     for (int i = 0; i < n; ++i) stdg::join(total, low, x[i]);
@@ -32,6 +47,8 @@ def lib(tmp_path_factory):
     out = ctypes.CDLL(str(d / "sums.so"))
     out.joined.restype = ctypes.c_float
     out.joined.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    out.row_sum.restype = ctypes.c_float
+    out.row_sum.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     return out
 
 
@@ -53,3 +70,25 @@ def test_infinite_total_stays_infinite(lib):
         assert lib.joined(x.ctypes.data, x.size) == want
     x = np.array([np.inf, -np.inf, 1.0], dtype=np.float32)
     assert np.isnan(lib.joined(x.ctypes.data, 3))
+
+
+@pytest.mark.parametrize("slots,n", [(4, 6), (4, 12), (4, 30), (5, 12), (5, 60)])
+def test_row_sum_of_conjugate_gradients(lib, slots, n):
+    # the operator row inside the fused CG kernels: root mean square error over random rows at most 0.9 of that of plain
+    # FP32 totals of chains of 10 or 6 products (0.7 to 0.85 expected; 1 without the compensation)
+    rng = np.random.default_rng(n)
+    rows, ch = 4000, 10 if n % 10 == 0 else 6
+    K, X = rng.normal(size=(2, rows, slots * n)).astype(np.float32)
+    exact = np.sum(K.astype(np.float64) * X, axis=1)
+    got = np.array([lib.row_sum(k.ctypes.data, x.ctypes.data, slots, n) for k, x in zip(K, X)], dtype=np.float64)
+    total = np.zeros(rows, dtype=np.float32)
+    for s in range(slots):
+        slot = np.zeros(rows, dtype=np.float32)
+        for c in range(s * n, (s + 1) * n, ch):
+            chain = np.zeros(rows, dtype=np.float32)
+            for j in range(c, c + ch):
+                chain = (K[:, j].astype(np.float64) * X[:, j] + chain).astype(np.float32)
+            slot += chain
+        total += slot
+    rms = lambda e: np.sqrt(np.mean(e ** 2))  # noqa: E731
+    assert rms(got - exact) < 0.9 * rms(total.astype(np.float64) - exact)
