@@ -25,6 +25,24 @@ STDG_HD void join(float& total, float& low, float sum) {
 // the collected errors, to be added to the total last (none where the total is not finite)
 STDG_HD float rest(float total, float low) { return total - total == 0.f ? low : 0.f; }
 
+// Three floats whose sum is the value.  Additions carry the rounding errors of the two leading terms on
+// (Knuth's two-sum), so that a tree over 32 lanes errs by some 2^-70 of the magnitudes: below an FP64 tree,
+// without its arithmetic (an FP64 instruction takes 16 cycles of the SM).  The leading terms must not overflow
+// in the sum: kTripleMax each for 32 of them.
+constexpr float kTripleMax = 5.3e36f;
+struct Triple {
+    float s, c, d;
+    STDG_HD void plus(const Triple& o) {
+        const float a = s + o.s, av = a - s, ae = (s - (a - av)) + (o.s - av);
+        const float b = c + o.c, bv = b - c, be = (c - (b - bv)) + (o.c - bv);
+        const float g = b + ae, gv = g - b, ge = (b - (g - gv)) + (ae - gv);
+        s = a;
+        c = g;
+        d += o.d + (be + ge);
+    }
+    STDG_HD double value() const { return (double)s + ((double)c + (double)d); }
+};
+
 // Sum of a row's products over the couplings, CH columns at a time.  FP64: a chain per neighbour, then their
 // sum.  FP32: as the operator by itself (coupling_apply.h), chains of half as many columns joined with
 // compensation; plain totals had 4% (2D p = 1) to 7% (3D p = 1) more error than the face form's.

@@ -5,6 +5,8 @@
 
 #include <cstdint>
 
+#include "compensated.h"
+
 namespace stdg {
 
 constexpr int kMaxRestart = 64;
@@ -99,15 +101,16 @@ template <> struct Acc<float> {
         c += te + pe;
     }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-    // adds the pair `give` of lane ^ o (TwoSum of the leading terms): the tree over the lanes stays in
-    // float pairs, because at two FP64 lanes an SM the conversions and FP64 additions of 16 sums per
-    // thread took 5 us a block, more than the products
+};
+// FP32 accumulators in the tree over the lanes.  At two FP64 lanes an SM the conversions and FP64
+// additions of 16 sums per thread took 5 us a block, more than the products; three floats lose no
+// bit of an FP64 tree (compensated.h)
+template <> struct Acc<Triple> {
+    Triple t;
+    __device__ __forceinline__ double value() const { return t.value(); }
     __device__ __forceinline__ void plus_xor(const Acc& give, int o) {
-        const float os = __shfl_xor_sync(0xffffffffu, give.s, o), oc = __shfl_xor_sync(0xffffffffu, give.c, o);
-        const float t = s + os;
-        const float z = t - s;
-        c += oc + ((s - (t - z)) + (os - z));
-        s = t;
+        t.plus(Triple{__shfl_xor_sync(0xffffffffu, give.t.s, o), __shfl_xor_sync(0xffffffffu, give.t.c, o),
+                      __shfl_xor_sync(0xffffffffu, give.t.d, o)});
     }
 };
 
@@ -125,13 +128,14 @@ __device__ __forceinline__ bool last_block(unsigned* counter, unsigned total) {
     return last;
 }
 
-// Block-wide sums of the 16 accumulators that each thread holds: the lanes of a warp halve their
-// set at every exchange (16 exchanges instead of 80), then FP64 sums over the warps through shared
-// memory.  The sum of accumulator k is valid in thread k < 16.
+// Sums over the lanes of a warp of the 16 accumulators that each thread holds: the lanes halve their set at
+// every exchange (16 exchanges instead of 80).  Lanes 2 i and 2 i + 1 end with the sum of accumulator
+// lane_of16(lane).
+__device__ __forceinline__ int lane_of16(int lane) {
+    return (lane & 16 ? 8 : 0) + (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+}
 template <typename R>
-__device__ __forceinline__ double block_sum16(Acc<R> (&v)[kDotChunk]) {
-    __shared__ double red[32][kDotChunk];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ double lane_sums16(Acc<R> (&v)[kDotChunk], int lane) {
 #pragma unroll
     for (int o = 16, n = kDotChunk / 2; o > 1; o >>= 1, n >>= 1) {
         const bool up = lane & o;
@@ -143,9 +147,33 @@ __device__ __forceinline__ double block_sum16(Acc<R> (&v)[kDotChunk]) {
         }
     }
     v[0].plus_xor(v[0], 1);
-    const int k = (lane & 16 ? 8 : 0) + (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+    return v[0].value();
+}
+__device__ __forceinline__ double lane_sums16(Acc<float> (&v)[kDotChunk], int lane) {
+    bool fits = true;
+#pragma unroll
+    for (int k = 0; k < kDotChunk; ++k) fits = fits && fabsf(v[k].s) <= kTripleMax;
+    if (__all_sync(0xffffffffu, fits)) {
+        Acc<Triple> t[kDotChunk];
+#pragma unroll
+        for (int k = 0; k < kDotChunk; ++k) t[k].t = Triple{v[k].s, v[k].c, 0.f};
+        return lane_sums16<Triple>(t, lane);
+    }
+    Acc<double> t[kDotChunk];   // values that FP32 cannot add, infinities and NaN
+#pragma unroll
+    for (int k = 0; k < kDotChunk; ++k) t[k].s = v[k].value();
+    return lane_sums16<double>(t, lane);
+}
+
+// Block-wide sums of the 16 accumulators: over the lanes, then FP64 sums over the warps through shared
+// memory.  The sum of accumulator k is valid in thread k < 16.
+template <typename R>
+__device__ __forceinline__ double block_sum16(Acc<R> (&v)[kDotChunk]) {
+    __shared__ double red[32][kDotChunk];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double mine = lane_sums16(v, lane);
     __syncthreads();
-    if ((lane & 1) == 0) red[warp][k] = v[0].value();
+    if ((lane & 1) == 0) red[warp][lane_of16(lane)] = mine;
     __syncthreads();
     double s = 0;
     if (threadIdx.x < kDotChunk)
@@ -153,15 +181,26 @@ __device__ __forceinline__ double block_sum16(Acc<R> (&v)[kDotChunk]) {
     return s;
 }
 
+// Sum of one accumulator over the lanes of a warp.
+template <typename R>
+__device__ __forceinline__ double lane_sum1(Acc<R> v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v.plus_xor(v, o);
+    return v.value();
+}
+__device__ __forceinline__ double lane_sum1(Acc<float> v) {
+    if (__all_sync(0xffffffffu, fabsf(v.s) <= kTripleMax)) return lane_sum1<Triple>(Acc<Triple>{{v.s, v.c, 0.f}});
+    return lane_sum1<double>(Acc<double>{v.value()});
+}
+
 // Block-wide sum of one accumulator; valid in thread 0.
 template <typename R>
 __device__ __forceinline__ double block_sum1(Acc<R> v) {
     __shared__ double red[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v.plus_xor(v, o);
+    const double mine = lane_sum1(v);
     __syncthreads();
-    if (lane == 0) red[warp] = v.value();
+    if (lane == 0) red[warp] = mine;
     __syncthreads();
     double s = 0;
     if (threadIdx.x == 0)

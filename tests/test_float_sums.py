@@ -27,6 +27,13 @@ template <int CH> static float row(const float* k, const float* x, int slots, in
 extern "C" float row_sum(const float* k, const float* x, int slots, int n) {
     return n % 10 == 0 ? row<10>(k, x, slots, n) : row<6>(k, x, slots, n);
 }
+extern "C" double tree(const float* s, const float* c) {   // 32 lanes, as the butterfly adds them in lane 0
+    stdg::Triple v[32];
+    for (int i = 0; i < 32; ++i) v[i] = stdg::Triple{s[i], c[i], 0.f};
+    for (int o = 16; o > 0; o >>= 1)
+        for (int i = 0; i < o; ++i) v[i].plus(v[i + o]);
+    return v[0].value();
+}
 extern "C" float joined(const float* x, int n) {
     float total = 0.f, low = 0.f;
     for (int i = 0; i < n; ++i) stdg::join(total, low, x[i]);
@@ -49,6 +56,8 @@ def lib(tmp_path_factory):
     out.joined.argtypes = [ctypes.c_void_p, ctypes.c_int]
     out.row_sum.restype = ctypes.c_float
     out.row_sum.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    out.tree.restype = ctypes.c_double
+    out.tree.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
     return out
 
 
@@ -92,3 +101,21 @@ def test_row_sum_of_conjugate_gradients(lib, slots, n):
         total += slot
     rms = lambda e: np.sqrt(np.mean(e ** 2))  # noqa: E731
     assert rms(got - exact) < 0.9 * rms(total.astype(np.float64) - exact)
+
+
+@pytest.mark.parametrize("cancel", [False, True])
+@pytest.mark.parametrize("scale", [1.0, 1e30, 1e-30])
+def test_lane_tree_loses_no_bit_of_fp64(lib, cancel, scale):
+    # FP32 inner products reach the tree over the lanes as pairs s + c, |c| some 2^-24 |s|. Its result is the exact sum
+    # rounded to FP64, up to 2^-68 of the magnitudes (six additions of third terms at 2^-24 of 2^-48 each, with room) and
+    # the smallest subnormal
+    rng = np.random.default_rng(5)
+    for _ in range(200):
+        s = (scale * rng.normal(size=32) * 2.0 ** rng.integers(-6, 7, 32)).astype(np.float32)
+        if cancel:
+            s[16:] = -s[:16]
+        c = (s * 2.0 ** -24 * rng.uniform(-8, 8, 32)).astype(np.float32)
+        exact = sum(Fraction(float(v)) for v in s) + sum(Fraction(float(v)) for v in c)
+        got = Fraction(lib.tree(s.ctypes.data, c.ctypes.data))
+        mag = sum(abs(Fraction(float(v))) for v in s)
+        assert abs(got - exact) <= abs(exact) * Fraction(2) ** -52 + mag * Fraction(2) ** -68 + 64 * Fraction(2) ** -149
