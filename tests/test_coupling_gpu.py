@@ -259,3 +259,31 @@ def test_fp32_results_that_overflow_are_infinite(dim, p):
     big, small = np.abs(ref) > 1e39, np.abs(ref) < 1e38 * w.dt ** 2 / 4
     assert big.any() and np.array_equal(y[big], np.sign(ref[big]) * np.inf)
     assert np.isfinite(y[small]).all()
+
+
+@pytest.mark.parametrize("shots", [19, 20, 21, 33, 64])
+def test_stacked_shots_from_the_face_blocks(shots):
+    # without the couplings, batches around the 20 shots from which a lane takes a shot, and around its 32 lanes
+    need_gpu()
+    w = _workload(2, 2, 2, n=3)
+    rng = np.random.default_rng(shots)
+    out = []
+    for share in (0.0, 1.0):
+        s = _solver(w, precision="mixed", preconditioner=1, rel_tol=1e-11, max_iters=20000)
+        s.set_coupling_share(share)
+        s.set_material(w.lam, w.mu, w.rho)
+        assert (s.coupling_bytes > 0) == (share > 0)
+        s.set_shots(shots)
+        v0, sig0 = s.get_state(0)
+        if not out:
+            states = [(rng.normal(size=v0.shape), rng.normal(size=sig0.shape)) for _ in range(shots)]
+        for k, st in enumerate(states):
+            s.set_state(*st, shot=k)
+        s.step(w.dt, 1)
+        out.append(np.array([s.get_state(k)[0] for k in range(shots)]))
+    for k in range(shots):
+        assert rel_l2(out[0][k], out[1][k]) < 1e-8
+    sim = oracle_sim(w)
+    sim.set_state(*states[-1])
+    sim.step(1)
+    assert rel_l2(out[0][-1], sim.v_tr) < 1e-8
