@@ -283,7 +283,7 @@ int stdg_apply_preconditioner(stdg_ctx* ctx, double dt, const double* r, double*
  * velocity values per slab, canonical layout), on device buffers owned by the caller (r_dev
  * and z_dev distinct), slab size dt.  fp32 = 0: the FP64 preconditioner of the FP64 solver;
  * fp32 != 0 (mixed-precision contexts only): the FP32 one of the inner solve -- for the stencil
- * preconditioner with more than 24 shots and d N_phi N_gamma = 36, its element-local step runs on
+ * preconditioner with 25 shots or more and d N_phi N_gamma = 36, its element-local step runs on
  * the tensor cores (kind::tf32 with S^{-1} rounded to TF32 and the vector split into two TF32
  * terms).  Appendix A, Eq. pre1 (Pre1) or Eqs. APPRE1-APPRE2 (Pre2).  Synchronises the stream;
  * STDG_ESTATE without a preconditioner or shots, STDG_ECUDA if a bounded wait gave up. */

@@ -124,6 +124,17 @@ void source_basis_host(const stdg_ctx* c, int64_t q, double* phi, double* dphi) 
     }
 }
 
+// Tensor-core image of the FP32 stencil blocks: held while the context has the shots that use it.
+static int fit_mma_image(stdg_ctx* c) {
+    const bool want = c->d_pre2_32 && pre2_mma_supported(c) && c->n_shots >= kMmaShots;
+    if (want == (c->d_pre2_mma != nullptr)) return STDG_OK;
+    c->mma_dt = -1.0;
+    if (want) return dev_alloc(c, (void**)&c->d_pre2_mma, sizeof(float) * pre2_mma_image_floats(c));
+    dev_free(c, c->d_pre2_mma);
+    c->d_pre2_mma = nullptr;
+    return STDG_OK;
+}
+
 static int alloc_state(stdg_ctx* c, int n_shots) {
     dev_free(c, c->d_vtr);
     dev_free(c, c->d_sigtr);
@@ -149,6 +160,7 @@ static int alloc_state(stdg_ctx* c, int n_shots) {
     c->n_shots = n_shots;
     c->rec_steps = 0;
     solver_invalidate_graph(c);
+    if ((rc = fit_mma_image(c)) != STDG_OK) return rc;
     return solver_setup(c);   // stacked Krylov workspace sized for n_shots
 }
 
@@ -260,9 +272,6 @@ static int setup_pre1(stdg_ctx* c) {
                 (rc = dev_alloc(c, (void**)&c->d_pre2, sizeof(double) * nS)) != STDG_OK) return rc;
             if (c->opt.precision != STDG_FP64 &&
                 (rc = dev_alloc(c, (void**)&c->d_pre2_32, sizeof(float) * ne * pre2_stride32(c))) != STDG_OK) return rc;
-            // tensor-core image of the FP32 blocks for batches of shots
-            if (c->opt.precision != STDG_FP64 && pre2_mma_supported(c) &&
-                (rc = dev_alloc(c, (void**)&c->d_pre2_mma, sizeof(float) * pre2_mma_image_floats(c))) != STDG_OK) return rc;
             // FP16 balanced copy for one shot (the dominant stream at half the bytes)
             if (c->opt.precision != STDG_FP64 && pre2_half_supported(c)) {
                 if ((rc = dev_alloc(c, &c->d_pre2_16, 2 * (size_t)ne * N * N)) != STDG_OK) return rc;
@@ -270,6 +279,7 @@ static int setup_pre1(stdg_ctx* c) {
             }
             if ((rc = dev_alloc(c, (void**)&c->d_p2status, sizeof(int))) != STDG_OK) return rc;
         }
+        if ((rc = fit_mma_image(c)) != STDG_OK) return rc;
     }
     c->pre_dt = -1.0;
     return STDG_OK;
@@ -278,13 +288,16 @@ static int setup_pre1(stdg_ctx* c) {
 // Time blocks of the block-Jacobi preconditioner and, for the stencil preconditioner, the
 // local Schur-complement inverses, for slab size dt (rebuilt only when dt changes).
 int precond_for_dt(stdg_ctx* c, double dt) {
-    if (!c->opt.preconditioner || c->pre_dt == dt) return STDG_OK;
-    STDG_CUDA(c, launch_pre1_time(c, dt));
-    c->pre_dt = dt;
-    if (c->opt.preconditioner == 2) {
+    if (!c->opt.preconditioner) return STDG_OK;
+    const bool fresh = c->pre_dt != dt;
+    if (fresh) {
+        STDG_CUDA(c, launch_pre1_time(c, dt));
+        c->pre_dt = dt;
+        c->mma_dt = -1.0;
+    }
+    if (fresh && c->opt.preconditioner == 2) {
         STDG_CUDA(c, cudaMemsetAsync(c->d_p2status, 0, sizeof(int), c->stream));
         STDG_CUDA(c, launch_pre2_setup(c, dt, c->d_p2status));
-        if (c->d_pre2_mma) STDG_CUDA(c, launch_pre2_mma_image(c));
         if (c->d_pre2_16) STDG_CUDA(c, launch_pre2_half(c));
         int status = 0;
         STDG_CUDA(c, cudaMemcpyAsync(&status, c->d_p2status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -293,6 +306,10 @@ int precond_for_dt(stdg_ctx* c, double dt) {
             c->pre_dt = -1.0;
             STDG_FAIL(c, STDG_ECUDA, "stencil preconditioner: a local Schur complement is singular");
         }
+    }
+    if (c->d_pre2_mma && c->mma_dt != dt) {
+        STDG_CUDA(c, launch_pre2_mma_image(c));
+        c->mma_dt = dt;
     }
     return STDG_OK;
 }
@@ -433,6 +450,7 @@ int stdg_set_mesh(stdg_ctx* c, int64_t n_vert, const double* xyz, int64_t n_elem
     c->d_pre2 = nullptr;
     c->d_pre2_32 = nullptr;
     c->d_pre2_mma = nullptr;
+    c->mma_dt = -1.0;
     c->d_pre2_16 = nullptr;
     c->d_pre2_scl = nullptr;
     c->d_p2y = c->d_p2t = nullptr;

@@ -378,7 +378,7 @@ cudaError_t launch_pre2_mma_image(stdg_ctx* c) {
 bool launch_pre2_local_mma(stdg_ctx* c, const float* r, const int* ridx, int64_t ld, const float* w, float* z,
                            int nshots, cudaError_t* e) {
     using Sh = MmaShape<36>;
-    if (!pre2_mma_supported(c) || !c->d_pre2_mma || nshots < 2 || !c->d_err) return false;
+    if (!pre2_mma_supported(c) || !c->d_pre2_mma || !c->d_err) return false;
     const bool aligned = (reinterpret_cast<uintptr_t>(r) % 16 == 0) && (reinterpret_cast<uintptr_t>(w) % 16 == 0) &&
                          (reinterpret_cast<uintptr_t>(z) % 16 == 0) && (ld % 4 == 0) && (c->nvel % 4 == 0);
     if (!aligned) return false;

@@ -496,9 +496,7 @@ static cudaError_t pre2_local_t(stdg_ctx* c, const R* Sinv, int64_t es, const R*
     const int N = c->dim * c->Nphi * c->Ng;
     if constexpr (std::is_same<R, float>::value) {   // a batch of shots: one GEMM per element pair on the tensor cores
         cudaError_t e;
-        // up to 24 shots the FP32 blocks are faster (6,400 triangles, p = 2: 8 shots 17 against 51 us, 24 shots
-        // 44 against 54 us, 32 shots 58 against 55 us; the same order at 1,600 and 25,600) and not rounded to TF32
-        if (nshots > 24 && launch_pre2_local_mma(c, r, ridx, ld, w, z, nshots, &e)) return e;
+        if (nshots >= kMmaShots && launch_pre2_local_mma(c, r, ridx, ld, w, z, nshots, &e)) return e;
     }
     if constexpr (std::is_same<R, float>::value) {
         const int wpb = c->tune.pre2_wpb;

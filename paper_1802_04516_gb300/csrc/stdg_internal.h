@@ -162,7 +162,8 @@ struct stdg_ctx {
     // ---- stencil preconditioner (precond2.cu): S_i^{-1} per element, column-major
     double* d_pre2 = nullptr;
     float* d_pre2_32 = nullptr;                // FP32 copy for the FP32 solver, pre2_stride32 apart
-    float* d_pre2_mma = nullptr;               // TF32-rounded tensor-core operand image (multi-shot, pre2_mma.cu)
+    float* d_pre2_mma = nullptr;               // TF32-rounded tensor-core operand image (kMmaShots shots or more, pre2_mma.cu)
+    double mma_dt = -1.0;                      // slab size that the image was made for
     void* d_pre2_16 = nullptr;                 // FP16 balanced blocks H (S^-1 = diag(r) H diag(c)), single shot
     float* d_pre2_scl = nullptr;               // per element: row scales r then column scales c
     int pre2_bits = 16;                        // storage of the FP32 path's local blocks: 16 or 32
@@ -293,6 +294,10 @@ cudaError_t launch_pre2_apply32(stdg_ctx* c, const float* r, float* z, const int
 cudaError_t launch_pre2_local(stdg_ctx* c, int fp32, const void* r, const void* w, void* z);
 cudaError_t launch_pre2_local_batch(stdg_ctx* c, const float* r, const float* w, float* z);
 // pre2_mma.cu: the element-local step for a batch of shots on the tensor cores (tcgen05)
+// Fewest shots that take it: up to 24 the FP32 blocks are faster (6,400 triangles, p = 2: 8 shots 17 against
+// 51 us, 24 shots 44 against 54 us, 32 shots 58 against 55 us; the same order at 1,600 and 25,600) and not
+// rounded to TF32
+constexpr int kMmaShots = 25;
 bool pre2_mma_supported(const stdg_ctx* c);
 int64_t pre2_mma_image_floats(const stdg_ctx* c);
 cudaError_t launch_pre2_mma_image(stdg_ctx* c);
