@@ -352,18 +352,21 @@ typedef struct {
     int face_warps_per_block;   /* face kernels of the operator: warps per block (1, 2, 4)            */
     int face_blocks_per_sm;     /* single-shot bulk-copy face kernel: grid cap, blocks per SM         */
     int face_register_cap;      /* single-shot bulk-copy face kernel: 1 register cap for occupancy, 0 none */
-    int pre2_warps_per_block;   /* CUDA-core element-local step of the stencil preconditioner         */
-    int mma_ctas_per_sm;        /* tensor-core element-local step (a batch of shots): CTAs per SM (1, 2) */
-    double face_ms, pre2_ms;    /* best time per launch of the tuned face kernel / local step (0: not tuned) */
+    int pre2_warps_per_block;   /* stencil preconditioner's element-local step of one shot, 16-bit blocks */
+    int mma_ctas_per_sm;        /* tensor-core element-local step (25 shots or more): CTAs per SM (1, 2) */
+    double face_ms, pre2_ms;    /* best time of the operator from the FP32 face blocks / of the local step (0: not run) */
     int candidates;             /* configurations timed                                               */
 } stdg_tuning;
 
 /* Autotuner: times every candidate launch shape of the hot kernels this context runs for slab
  * size dt -- the FP32 face kernel (mixed precision; warps per block 1/2/4 and, for one shot, the
- * grid cap 8/16/32/64 blocks per SM and the kernel compiled with or without a register cap) and the element-local step of the stencil preconditioner
- * (warps per block, or CTAs per SM of the tensor-core kernel) -- on the context's own mesh and
+ * grid cap 8/16/32/64 blocks per SM and the kernel compiled with or without a register cap) and the
+ * element-local step of the stencil preconditioner (warps per block with the 16-bit blocks of one
+ * shot, CTAs per SM of the tensor-core kernel) -- on the context's own mesh and
  * shot count (zero vectors, 10 launches each, CUDA events) and keeps the fastest for every later
- * launch; step graphs captured before are dropped and re-captured.  `out` (may be NULL) receives
+ * launch; a setting that the kernel in use does not read stays as it is, and a kernel without
+ * settings is timed once.  The element couplings have none: where they are kept, the face kernel's
+ * settings serve once they are given back.  Step graphs captured before are dropped and re-captured.  `out` (may be NULL) receives
  * the choices.  Allocates three scratch vectors for the call.  Results do not depend on the
  * choice beyond the order of floating-point atomics. */
 int stdg_autotune(stdg_ctx* ctx, double dt, stdg_tuning* out);

@@ -1198,20 +1198,20 @@ int stdg_autotune(stdg_ctx* c, double dt, stdg_tuning* out) {
         return ms / n;
     };
     stdg_tuning res{};
-    // the face kernel of the Krylov operator: FP32 in mixed precision (the bulk-copy kernel for one
-    // shot, the register kernel for a batch), FP64 otherwise (its generic kernel has fixed shapes)
+    // the operator from the FP32 face blocks (also where the couplings are kept, which have no such settings:
+    // the face kernels take over when those are given back), over the settings that its kernel reads: all of
+    // them for one shot, the warps per block for a batch, none in the generic kernel or in FP64
     if (mixed) {
         double best = 1e30;
         Tuning bt = c->tune;
-        for (int cap : (ns == 1 ? std::vector<int>{1, 0} : std::vector<int>{1}))
-            for (int wpb : {1, 2, 4})
-                for (int bpsm : (ns == 1 ? std::vector<int>{8, 16, 32, 64} : std::vector<int>{16})) {
+        const bool fast = face_fast_shape(c), one = fast && ns == 1;
+        for (int cap : (one ? std::vector<int>{1, 0} : std::vector<int>{bt.face_cap}))
+            for (int wpb : (fast ? std::vector<int>{1, 2, 4} : std::vector<int>{bt.face_wpb}))
+                for (int bpsm : (one ? std::vector<int>{8, 16, 32, 64} : std::vector<int>{bt.face_bpsm})) {
                     c->tune.face_cap = cap;
                     c->tune.face_wpb = wpb;
                     c->tune.face_bpsm = bpsm;
-                    const double ms = time([&]() {
-                        return launch_apply32(c, dt, (const float*)dx, (float*)dy, 1.0, nullptr, 0, ns);
-                    });
+                    const double ms = time([&]() { return launch_apply_faces32(c, dt, (const float*)dx, (float*)dy, ns); });
                     if (ms < best) { best = ms; bt = c->tune; }
                 }
         c->tune = bt;
@@ -1220,9 +1220,12 @@ int stdg_autotune(stdg_ctx* c, double dt, stdg_tuning* out) {
     if (c->opt.preconditioner == 2) {
         double best = 1e30;
         Tuning bt = c->tune;
-        const bool mma = mixed && ns > 1 && c->d_pre2_mma;
-        for (int k : (mma ? std::vector<int>{1, 2} : std::vector<int>{1, 2, 4})) {
-            if (mma) c->tune.mma_cps = k; else c->tune.pre2_wpb = k;
+        // the tensor-core kernel reads the CTAs per SM, the kernel of the 16-bit blocks of one shot its warps per
+        // block; the others have fixed shapes and are timed once
+        const bool mma = mixed && ns >= kMmaShots && c->d_pre2_mma, half = mixed && ns == 1 && c->d_pre2_16 && c->pre2_bits == 16;
+        for (int k : (mma ? std::vector<int>{1, 2} : half ? std::vector<int>{1, 2, 4} : std::vector<int>{0})) {
+            if (mma) c->tune.mma_cps = k;
+            if (half) c->tune.pre2_wpb = k;
             const double ms = time([&]() -> cudaError_t {
                 if (mixed) return launch_pre2_local_batch(c, (const float*)dx, (const float*)dw, (float*)dy);
                 return launch_pre2_local(c, 0, dx, dw, dy);

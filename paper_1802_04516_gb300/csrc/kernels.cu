@@ -821,12 +821,21 @@ bool coupling32_wanted(const stdg_ctx* c) {
     return !(c->dim == 3 && c->Ng == 1 && (int64_t)sizeof(float) * n2 * (2 * c->n_face + c->n_elem) > (80LL << 20));
 }
 
+// the operator from the face blocks, FP32
+static cudaError_t apply_faces32(stdg_ctx* c, const float* x, float* y, double scale, const int* xidx, int64_t ld, int nshots) {
+    STDG_DISPATCH(c->dim, c->Nphi, return (apply_tmpl<D_, N_, float>(c, c->d_D32, c->d_lamf32, c->d_muf32, c->d_rhoJ32, x, y, scale, true, true, xidx, ld, nshots)));
+    return cudaSuccess;
+}
+
 cudaError_t launch_apply32(stdg_ctx* c, double dt, const float* x, float* y, double cfac, const int* xidx, int64_t ld,
                            int nshots) {
     const double scale = cfac * schur_c(c) * dt * dt;
     if (c->d_Kf32) return launch_coupling32(c, x, xidx, ld, nullptr, nullptr, 0, y, scale, nshots);
-    STDG_DISPATCH(c->dim, c->Nphi, return (apply_tmpl<D_, N_, float>(c, c->d_D32, c->d_lamf32, c->d_muf32, c->d_rhoJ32, x, y, scale, true, true, xidx, ld, nshots)));
-    return cudaSuccess;
+    return apply_faces32(c, x, y, scale, xidx, ld, nshots);
+}
+
+cudaError_t launch_apply_faces32(stdg_ctx* c, double dt, const float* x, float* y, int nshots) {
+    return apply_faces32(c, x, y, schur_c(c) * dt * dt, nullptr, 0, nshots);
 }
 
 cudaError_t launch_apply_pre1(stdg_ctx* c, double dt, const double* y, const double* base, const int* bidx, int64_t bld,

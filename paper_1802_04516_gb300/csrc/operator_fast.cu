@@ -1271,6 +1271,9 @@ static cudaError_t launch_fast(stdg_ctx* c, const R* D, const R* lamf, const R* 
 static bool tiled2(const stdg_ctx* c) { return c->dim == 2 && c->Nphi == 10 && c->Ng == 4; }
 static bool tiled3(const stdg_ctx* c) { return c->dim == 3 && c->Nphi == 10 && c->Ng == 3; }
 bool face_tiled_shape(const stdg_ctx* c) { return tiled2(c) || tiled3(c); }
+bool face_fast_shape(const stdg_ctx* c) {
+    return tiled2(c) || tiled3(c) || (c->dim == 2 && ((c->Nphi == 6 && c->Ng == 3) || (c->Nphi == 3 && c->Ng == 1)));
+}
 int64_t face_tiled_floats(const stdg_ctx* c) {
     return tiled2(c) ? c->n_face * FaceTile::DT : tiled3(c) ? c->n_face * FaceTile3::DT : 0;
 }

@@ -221,6 +221,7 @@ cudaError_t launch_orthonormalize(stdg_ctx* c);
 cudaError_t launch_sig_convert(stdg_ctx* c, const double* in, double* out, int dir);
 cudaError_t launch_to_fp32(stdg_ctx* c);
 bool face_tiled_shape(const stdg_ctx* c);
+bool face_fast_shape(const stdg_ctx* c);     // FP32 face kernel with compile-time sizes
 int64_t face_tiled_floats(const stdg_ctx* c);
 cudaError_t launch_tile_d32(stdg_ctx* c);
 // y = A x (cfac scales the Schur part; 1 for the operator).  With xidx != null the input is
@@ -230,6 +231,8 @@ cudaError_t launch_apply(stdg_ctx* c, double dt, const double* x, double* y, dou
                          const int* xidx = nullptr, int64_t ld = 0, int nshots = 1);
 cudaError_t launch_apply32(stdg_ctx* c, double dt, const float* x, float* y, double cfac,
                            const int* xidx = nullptr, int64_t ld = 0, int nshots = 1);
+// y = A x from the face blocks whether or not the couplings are kept (autotuner)
+cudaError_t launch_apply_faces32(stdg_ctx* c, double dt, const float* x, float* y, int nshots);
 // y = A x (FP64, one shot) on the stream for a caller of the library.  While the caller records that stream
 // into a graph of its own the operator runs from the face blocks, which stay where they are until the next
 // mesh: the graph outlives this call, and the couplings may be given back before it is replayed

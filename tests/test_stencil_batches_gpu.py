@@ -1,7 +1,8 @@
 """The FP32 stencil preconditioner of stacked shots on both sides of the 25 shots from which its element-local step
 runs on the tensor cores (kind::tf32): below, the FP32 blocks at their own accuracy (1e-4, as the 32-bit blocks of
 one shot); from there on the TF32 blocks (2e-3), full and partial groups of shots, with the iteration counts and the
-convergence of FP32 blocks, on an image that only contexts with that many shots hold."""
+convergence of FP32 blocks, on an image that only contexts with that many shots hold; and the launch settings that the
+autotuner searches for each of these kernels."""
 import dataclasses
 
 import numpy as np
@@ -82,3 +83,24 @@ def test_tensor_core_blocks_converge_on_the_inversion_medium():
         assert st["status"] == 0
         worst = max(worst, st["iters_max"])
     assert worst < 400, worst
+
+
+@pytest.mark.parametrize("p,precision,pre,shots,face,local", [
+    (2, "mixed", 2, 1, 24, 3), (2, "mixed", 2, 9, 3, 1), (2, "mixed", 2, 29, 3, 2), (2, "fp64", 2, 1, 0, 1), (1, "mixed", 1, 1, 1, 0)])
+def test_autotuner_searches_what_the_kernels_read(p, precision, pre, shots, face, local):
+    # candidates: the face kernel's settings (the generic kernel of p = p_gamma = 1 has none) and the local step's; what
+    # is not searched keeps its default
+    need_gpu()
+    w = synth.scaled("c4", ny=8, p=p, steps=1, n_shots=shots)
+    s = gpu_solver(w, precision=precision, preconditioner=pre)
+    t = s.autotune(w.dt)
+    assert t["candidates"] == face + local
+    assert (t["face_ms"] > 0) == (face > 0) and (t["pre2_ms"] > 0) == (local > 0)
+    if face <= 3:
+        assert t["face_register_cap"] == 1 and t["face_blocks_per_sm"] == 16
+    if face <= 1:
+        assert t["face_warps_per_block"] == 4
+    if local != 3:
+        assert t["pre2_warps_per_block"] == 4
+    if local != 2:
+        assert t["mma_ctas_per_sm"] == 2
