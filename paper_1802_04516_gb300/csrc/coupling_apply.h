@@ -16,13 +16,20 @@ namespace stdg {
 // register.
 // FP64: bound by the pipe (an FP64 instruction takes 16 cycles of the SM however few lanes are
 // active), so a thread has one row and at most one lane in 16 is idle (17,956 triangles, p = 4,
-// p_gamma = 2: 642 us with the face and mass kernels, 406 us here; 40,000 at p = 2: 398 and 154 us).  K_ii and the r
+// p_gamma = 2: 642 us with the face and mass kernels, 410 us here; 40,000 at p = 2: 398 and 163 us).  K_ii and the r
 // side's K_lr^T are read by columns (consecutive across the threads), the l side's K_lr by pieces of
 // its rows; the two ways of loading differ between the elements of a warp, the products do not.
 // FP32: bound by L1 wavefronts, then by HBM.  A thread has two consecutive rows, so that one
 // 16-byte read of the staged values feeds them all, and the faces' blocks are kept in both
 // orientations, so that every load is a vector load of consecutive columns (reading rows of one copy
-// cost a wavefront per lane: 320 instead of 264 us on 200,704 triangles at p = 3).
+// cost a wavefront per lane).
+// Smooth vectors: the face term of a constant vanishes, which the face form sees before it multiplies by the
+// stiffness and the couplings only in the sum of their products.  So the value of the element's first node is
+// taken off its own and its neighbours' values, per component and time node, wherever every one of these
+// subtractions is exact; the mass term adds it again.  Otherwise (rough vectors, a change of binade) the values
+// stay as they are.  FP32 error on smooth vectors 1.1 to 2.0 times the face form's without this, 0.7 to 1.2 with
+// it, on constants 1.3 to 2.2 and 0.03 to 0.7; it costs 1 to 10% of a call (FP64 p = 4 on 17,956 triangles: 406 -> 410 us, p = 2 on 40,000
+// 163 -> 172 us; FP32 3D p = 3 on 7,986 tetrahedra 149 -> 153 us, p = 1 on 131,712 91 -> 102 us), 17% with one time node in FP32.
 // ---------------------------------------------------------------------------------
 template <typename R, int DIM, int NP, int NG, int SC>
 struct Coupling {
@@ -37,15 +44,36 @@ struct Coupling {
     static_assert(N % BL == 0 && BL % VJ == 0 && (CH == BL || (VJ == BL && VJ % CH == 0)), "chunks of whole loads");
     static_assert(N % 2 == 0, "d N_phi is even for every supported order");
     __host__ __device__ static constexpr int slots(bool own) { return FACES + (own ? 1 : 0); }
-    static size_t smem(int EB, bool own) { return sizeof(R) * (size_t)SC * slots(own) * EB * N * NGP; }
+    static constexpr int KA = DIM * NG;                       // constants of an element
+    // resident blocks of 160 threads that the compiler has to leave registers for, one shot with the element's own
+    // block: as many as fit without spills, fewer where ten columns are loaded together (FP32 3D p = 2, p_gamma = 1 204 -> 162 us,
+    // p = 3, p_gamma = 2 211 -> 150 us against the compiler's own choice; at p = 1 and 2 the same limit costs 20 to 40%)
+    __host__ __device__ static constexpr int blocks() {
+        if (!BOTH) return NG == 1 ? 7 : NG == 2 ? 5 : NG == 3 ? 4 : 3;
+        if (NG == 5) return DIM == 2 && N == 30 ? 3 : 2;
+        return N % 10 == 0 || NG == 4 ? 3 : NG == 3 ? 5 : NG == 2 ? 6 : 8;
+    }
+    static size_t smem(int EB, bool own) {
+        return sizeof(R) * (size_t)SC * slots(own) * EB * N * NGP + (own ? (sizeof(R) + sizeof(int)) * (size_t)SC * EB * KA : 0);
+    }
 };
+
+// v - c is exact: c finite, v of the same sign and exponent (then c / 2 < v < 2 c, Sterbenz 1974)
+__device__ __forceinline__ bool exact_difference(float v, float c) {
+    const unsigned cb = __float_as_uint(c);
+    return (__float_as_uint(v) ^ cb) >> 23 == 0 && (cb & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool exact_difference(double v, double c) {
+    const unsigned cb = (unsigned)__double2hiint(c);
+    return ((unsigned)__double2hiint(v) ^ cb) >> 20 == 0 && (cb & 0x7ff00000u) != 0x7ff00000u;
+}
 
 template <typename R, int W> struct Piece;
 template <> struct Piece<float, 2> { using T = float2; };
 template <> struct Piece<double, 2> { using T = double2; };
 
 template <typename R, int DIM, int NP, int NG, int SC, bool OWN>
-__global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int EB, const int2* __restrict__ adj,
+__global__ void __launch_bounds__(OWN && SC == 1 ? 160 : 256, OWN && SC == 1 ? Coupling<R, DIM, NP, NG, SC>::blocks() : 0) coupling_apply_kernel(int64_t n_elem, int EB, const int2* __restrict__ adj,
                                                              const R* __restrict__ Ke, const R* __restrict__ Kf,
                                                              const R* __restrict__ rhoJ, const RefTables* __restrict__ rtp,
                                                              const R* __restrict__ x, const int* __restrict__ xidx, int64_t ld,
@@ -57,14 +85,19 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
     constexpr int SLOTS = C::slots(OWN), OFF = OWN ? 1 : 0;   // slot 0: the element itself, unless a base vector stands for it
     using P = typename Piece<R, 2>::T;   // two rows of a column (FP32), two columns of a row (FP64)
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ R sM[OWN ? NP * NP : 1], sT[NG * NG], sS[NG * NG];
+    constexpr int KA = C::KA;
+    __shared__ R sM[OWN ? NP * NP : 1], sM1[OWN ? NP : 1], sT[NG * NG], sS[NG * NG];
     R* sx = reinterpret_cast<R*>(smraw);                      // [shot of the chunk][slot][element][row (k,n)][time]
+    R* sc = sx + SC * SLOTS * EB * N * NGP;                   // [shot of the chunk][element][k][time]: the first node's value
+    int* sb = reinterpret_cast<int*>(sc + SC * EB * KA);      // the same: some subtraction would not be exact, nothing is taken off
     if (xidx) x += (int64_t)(*xidx) * ld;
     if (!OWN && bidx) base += (int64_t)(*bidx) * bld;
     const int64_t e0 = (int64_t)blockIdx.x * EB;
     const int ne = (int)min((int64_t)EB, n_elem - e0);
     if (OWN)
         for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sM[t] = (R)rtp->Mref[t];
+    if (OWN)
+        for (int t = threadIdx.x; t < NP; t += blockDim.x) sM1[t] = (R)rtp->Mrow[t];
     for (int t = threadIdx.x; t < NG * NG; t += blockDim.x) {
         if (OWN) sT[t] = (R)rtp->T[t];
         sS[t] = (R)(scale * rtp->S[t]);   // rounded once: its error is common to all elements
@@ -76,7 +109,19 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
     for (int i = 0; i < FACES; ++i) nb[i] = act ? adj[(e0 + le) * FACES + i] : make_int2(-1, 0);
     for (int s0 = 0; s0 < nshots; s0 += SC) {
         if (s0) __syncthreads();                              // the chunk before has been read
+        if (OWN) {
+            for (int t = threadIdx.x; t < SC * EB * KA; t += blockDim.x) sb[t] = 0;
+            __syncthreads();
+        }
         if (act) {   // the threads of an element stage its slots
+            static_assert(NV % TPE == 0, "a thread stages whole rounds of values");
+            constexpr int NVT = NV / TPE;
+            R first[SC == 1 ? NVT : 1];                       // of the values that the thread stages (one shot: loaded once)
+            unsigned rough[SC] = {};                          // bit i: a subtraction of value i's constant would round
+            if constexpr (OWN && SC == 1) {
+#pragma unroll
+                for (int i = 0; i < NVT; ++i) first[i] = x[(int64_t)s0 * nvec + (e0 + le) * NV + (i * TPE + row) / NP * NP];
+            }
 #pragma unroll
             for (int sl = 0; sl < SLOTS; ++sl) {
                 const int64_t e = sl < OFF ? e0 + le : nb[sl < OFF ? 0 : sl - OFF].x;
@@ -89,12 +134,40 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
 #pragma unroll
                     for (int t0 = 0; t0 < NV; t0 += TPE) {
                         const int t = t0 + row, ka = t / NP, nn = t % NP, k = ka / NG, a = ka % NG;
-                        if (NV % TPE == 0 || t < NV) dst[(k * NP + nn) * NGP + a] = src[t];
+                        const R v = src[t];
+                        dst[(k * NP + nn) * NGP + a] = v;
+                        if (OWN) {
+                            if (sl == 0 && nn == 0) sc[(c * EB + le) * KA + ka] = v;
+                            const R f = SC == 1 ? first[SC == 1 ? t0 / TPE : 0] : x[(int64_t)(s0 + c) * nvec + (e0 + le) * NV + ka * NP];
+                            rough[c] |= (exact_difference(v, f) ? 0u : 1u) << (t0 / TPE);
+                        }
                     }
                 }
             }
+            if (OWN) {
+#pragma unroll
+                for (int c = 0; c < SC; ++c)
+#pragma unroll
+                    for (int i = 0; i < NVT; ++i)
+                        if (rough[c] >> i & 1) sb[(c * EB + le) * KA + (i * TPE + row) / NP] = 1;
+            }
         }
         __syncthreads();
+        if (OWN) {
+            if (act) {
+#pragma unroll 1
+                for (int q = row; q < SC * NV; q += TPE) {
+                    const int c = q / NV, t = q % NV, ka = t / NP, nn = t % NP, k = ka / NG, a = ka % NG;
+                    const int at = (c * EB + le) * KA + ka;
+                    if (sb[at]) continue;
+                    const R off = sc[at];
+                    R* v = sx + (c * SLOTS * EB + le) * (N * NGP) + (k * NP + nn) * NGP + a;
+#pragma unroll
+                    for (int sl = 0; sl < SLOTS; ++sl) v[sl * EB * N * NGP] -= off;   // (slots of missing neighbours are not read)
+                }
+            }
+            __syncthreads();
+        }
         if (!act) continue;
         R bs[OWN || SC > 1 ? 1 : RPT][NG];   // the base values, loaded ahead of the sums
         if constexpr (!OWN && SC == 1) {
@@ -208,6 +281,11 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
                         for (int a = 0; a < NG; ++a) u[a] = fma(mv, xp[q * NGP + a], u[a]);
                     }
 #pragma unroll
+                    for (int a = 0; a < NG; ++a) {
+                        const int at = (c * EB + le) * KA + k * NG + a;
+                        u[a] = fma(sM1[nn], sb[at] ? (R)0 : sc[at], u[a]);
+                    }
+#pragma unroll
                     for (int a = 0; a < NG; ++a) u[a] *= rj;
                 }
 #pragma unroll
@@ -227,7 +305,7 @@ __global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t n_elem, int
 }
 
 // Elements per block: whole warps of threads (an idle lane costs as much as a busy one), at most
-// 128 threads and 48 KB, and at least one block per SM on small meshes.
+// 160 threads and 48 KB, and at least one block per SM on small meshes.
 template <typename R, int DIM, int NP, int NG, int SC, bool OWN>
 static cudaError_t coupling_go(stdg_ctx* c, const R* Ke, const R* Kf, const R* rhoJ, const R* x, const int* xidx, int64_t ld,
                                const R* base, const int* bidx, int64_t bld, R* y, double scale, int nshots) {

@@ -150,6 +150,10 @@ void build_ref_tables(int dim, int p, int pg, RefTables* rt) {
         for (int k = 0; k < n; ++k)
             for (int l = 0; l < n; ++l) rt->Mref[k * n + l] += q.wts[iq] * phi[k] * phi[l];
     }
+    for (int k = 0; k < n; ++k) {
+        rt->Mrow[k] = 0.0;
+        for (int l = 0; l < n; ++l) rt->Mrow[k] += rt->Mref[k * n + l];
+    }
     std::memcpy(rt->MrefInv, rt->Mref, sizeof(double) * n * n);
     invert(n, rt->MrefInv);
     {   // Cholesky factor R of M_ref and its inverse (lower triangular)

@@ -22,6 +22,7 @@ struct RefTables {
     int succ[kMaxNP][3];          // index of exps[b] + unit exponent s (-1 beyond degree p)
     double coef[kMaxNP * kMaxNP]; // phi_k(xi) = sum_a coef[a*Nphi + k] xi^a
     double Mref[kMaxNP * kMaxNP]; // int_{ref simplex} phi_k phi_m
+    double Mrow[kMaxNP];          // its row sums, int_{ref simplex} phi_k
     double MrefInv[kMaxNP * kMaxNP];
     double MrefLinv[kMaxNP * kMaxNP];   // R^{-1} with M_ref = R R^T (R lower triangular)
     double tnodes[kMaxNG], W[kMaxNG], g0[kMaxNG], g1[kMaxNG];

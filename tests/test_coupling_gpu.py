@@ -287,3 +287,42 @@ def test_stacked_shots_from_the_face_blocks(shots):
     sim.set_state(*states[-1])
     sim.step(1)
     assert rel_l2(out[0][-1], sim.v_tr) < 1e-8
+
+
+@pytest.mark.parametrize("dim,p,pg", [(2, 1, 0), (2, 2, 2), (2, 4, 2), (3, 1, 1), (3, 3, 3)])
+@pytest.mark.parametrize("shift", [0.0, 1e-3])
+def test_constant_and_nearly_constant_vectors_lose_nothing_to_cancellation(dim, p, pg, shift):
+    # the face term of a constant is zero: the operator leaves the mass term, a few roundings of each value (20 eps in
+    # FP64, 5 in FP32 in norm). A small rough part on top of the constant comes out as the operator on that part alone.
+    torch = need_gpu()
+    from paper_1802_04516_gb300 import binding
+    w = synth.scaled("c2", ny=10, p=p, steps=1) if dim == 2 else _workload(dim, p, pg)
+    w.p_gamma, w.scheme = pg, "cn" if pg == 0 else "stdg"
+    s = _solver(w, precision="mixed", preconditioner=0)
+    assert s.coupling_bytes > 0
+    NP, NG = s.query(2), s.query(4)
+    M, T = np.zeros((NP, NP)), np.zeros((NG, NG))
+    d = lambda a: a.ctypes.data_as(binding._D)  # noqa: E731
+    binding.load().stdg_reference_tables(dim, p, pg, d(M), None, d(T), None, None, None)
+    X = np.asarray(w.xyz)[w.elem_vert]
+    det = np.linalg.det(X[:, 1:] - X[:, :1])
+    rng = np.random.default_rng(4)
+    x = np.broadcast_to(rng.uniform(1.1, 1.9, (1, dim, 1, 1)), (w.n_elem, dim, NG, NP)).astype(np.float32).astype(np.float64)
+    rough = (shift * rng.uniform(-1, 1, x.shape)).astype(np.float32).astype(np.float64)
+    full = (x + rough).astype(np.float32).astype(np.float64)   # stays within the binade 1..2
+    rough = full - x
+
+    def run(v, fp32):
+        if not fp32:
+            return s.apply_operator(w.dt, v.ravel()).reshape(v.shape)
+        vd = torch.tensor(v.ravel(), dtype=torch.float32, device="cuda")
+        yd = torch.zeros_like(vd)
+        torch.cuda.synchronize()
+        s.apply_operator_device(w.dt, vd.data_ptr(), yd.data_ptr(), fp32=True)
+        return yd.double().cpu().numpy().reshape(v.shape)
+
+    mass = np.einsum("e,ab,nm,ekbm->ekan", np.asarray(w.rho) * det, T, M, x)
+    exact = mass + (run(rough, False) if shift else 0.0)
+    for fp32, eps in ((False, 2.0 ** -53), (True, 2.0 ** -24)):
+        bar = (5 if fp32 else 20) * eps
+        assert rel_l2(run(full, fp32), exact) < bar
