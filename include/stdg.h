@@ -230,7 +230,7 @@ int stdg_query(stdg_ctx* ctx, int what, int64_t* out);
  * d N_phi N_gamma or above 128 keep FP32.  Returns STDG_OK or STDG_EINVAL (bits not 16/32). */
 int stdg_set_pre2_storage(stdg_ctx* ctx, int bits);
 
-/* Most of the device's free memory, 0 <= share <= 1 (default 1/16), that the operator's element
+/* Most of the device's free memory, 0 <= share <= 1 (default 1/6), that the operator's element
  * couplings may take when stdg_set_material or stdg_set_time_scale lays them out; what they leave
  * is there for other contexts, libraries and processes on the device, whose allocations cannot take
  * it back.  0 gives couplings that are held back at once and runs the operator from the face blocks.

@@ -329,7 +329,7 @@ class Solver:
 
     def set_coupling_share(self, share):
         """Most of the device's free memory that the operator's element couplings may take when the material is
-        set (default 1/16); 0 gives them back at once and runs the operator from the face blocks."""
+        set (default 1/6); 0 gives them back at once and runs the operator from the face blocks."""
         self._chk(self.lib.stdg_set_coupling_share(self.h, float(share)))
 
     coupling_bytes = property(lambda s: s.query(13))

@@ -179,7 +179,8 @@ static int ensure_fp32(stdg_ctx* c) {
 
 // Assembled couplings of the current medium (FP64, and their FP32 copy where D~ has one), where they
 // fit the share of the free memory that they may take.  Only this context can take their room back, so
-// the default share is small: the largest benchmark mesh (200,704 triangles, p = 3) needs 1.6 of 280 GB.
+// the default share is the least that the benchmarks use: 34 of some 230 GB free on 1,572,864 tetrahedra at p = 2
+// (200,704 triangles at p = 3 take 1.6 GB).
 static int setup_coupling(stdg_ctx* c) {
     const int64_t n2 = (int64_t)c->dim * c->Nphi * c->dim * c->Nphi, nKf = c->n_face * n2, nKe = c->n_elem * n2;
     const bool want32 = c->d_D32 != nullptr && coupling32_wanted(c);

@@ -10,9 +10,10 @@
 // take 23 us.  p' is read while p is written, so the two alternate between two buffers by iteration.
 // N_gamma = 1 throughout, so a row of an element is one value.
 //
-// Systems of up to 8,192 unknowns run in one cluster of 16 SMs for all their iterations: a thread per
+// Systems of up to 512 unknowns in whole elements per SM (8,192 in all; 8,160 or 7,680 where d N_phi does not
+// divide 512) run in one cluster of 16 SMs for all their iterations: a thread per
 // unknown keeps x, r, z, p and q in registers, only p crosses SMs (through L2), and the two reductions
-// of an iteration meet in distributed shared memory behind a cluster barrier, which costs less than the
+// of an iteration meet in distributed shared memory behind cluster barriers (three an iteration), which cost less than the
 // end of a kernel (9 us per iteration in the plane-wave problem).  Above that size 16 SMs are too few
 // (FP64 runs at two lanes an SM).
 #include <algorithm>
@@ -210,7 +211,6 @@ template <typename R, int DIM, int NP>
 struct CgRow {
     static constexpr int N = DIM * NP, SLOTS = DIM + 2;
     static constexpr bool KEEP = N <= 6;
-    static constexpr int THREADS = 512;
 };
 
 constexpr int kClusterSize = 16;

@@ -14,15 +14,16 @@ namespace stdg {
 // into shared memory as [row][time].  Thread (element, rows) forms the N_gamma sums of its rows for
 // SC shots at a time.  A value of K is used by one thread alone, so it goes straight from memory to a
 // register.
-// FP64: bound by the pipe (an FP64 instruction takes 16 cycles of the SM however few lanes are
+// FP64: bound by the pipe (0.97 busy at p = 4; an FP64 instruction takes 16 cycles of the SM however few lanes are
 // active), so a thread has one row and at most one lane in 16 is idle (17,956 triangles, p = 4,
 // p_gamma = 2: 642 us with the face and mass kernels, 410 us here; 40,000 at p = 2: 398 and 163 us).  K_ii and the r
 // side's K_lr^T are read by columns (consecutive across the threads), the l side's K_lr by pieces of
 // its rows; the two ways of loading differ between the elements of a warp, the products do not.
-// FP32: bound by L1 wavefronts, then by HBM.  A thread has two consecutive rows, so that one
-// 16-byte read of the staged values feeds them all, and the faces' blocks are kept in both
-// orientations, so that every load is a vector load of consecutive columns (reading rows of one copy
-// cost a wavefront per lane).
+// FP32: bound by the latency of K from memory (3D p = 3, 7,986 tetrahedra: 604 MB at 0.59 of the DRAM peak, 0.22 of the
+// warps resident, 7.7 of 9.9 cycles an instruction waits on a long scoreboard; L1 data pipe 0.39).  A thread has two
+// consecutive rows, so that one 16-byte read of the staged values feeds them all, and the faces' blocks are
+// kept in both orientations, so that every load is a vector load of consecutive columns (reading rows of
+// one copy cost a wavefront per lane).
 // Smooth vectors: the face term of a constant vanishes, which the face form sees before it multiplies by the
 // stiffness and the couplings only in the sum of their products.  So the value of the element's first node is
 // taken off its own and its neighbours' values, per component and time node, wherever every one of these
@@ -335,14 +336,21 @@ static cudaError_t coupling_ng(stdg_ctx* c, const R* Ke, const R* Kf, const R* r
                    : coupling_go<R, DIM, NP, NG, 4, true>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
 }
 
+// (the FP32 shapes with a tiled face kernel keep no FP32 couplings: coupling32_wanted)
 template <typename R, int DIM, int NP>
 static cudaError_t coupling_shape(stdg_ctx* c, const R* Ke, const R* Kf, const R* rhoJ, const R* x, const int* xidx, int64_t ld,
                                   const R* base, const int* bidx, int64_t bld, R* y, double scale, int ns) {
     switch (c->Ng) {
         case 1: return coupling_ng<R, DIM, NP, 1>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
         case 2: return coupling_ng<R, DIM, NP, 2>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
-        case 3: return coupling_ng<R, DIM, NP, 3>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
-        case 4: return coupling_ng<R, DIM, NP, 4>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
+        case 3:
+            if constexpr (sizeof(R) == 8 || DIM != 3 || NP != 10)
+                return coupling_ng<R, DIM, NP, 3>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
+            return cudaErrorInvalidValue;
+        case 4:
+            if constexpr (sizeof(R) == 8 || DIM != 2 || NP != 10)
+                return coupling_ng<R, DIM, NP, 4>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
+            return cudaErrorInvalidValue;
         case 5: return coupling_ng<R, DIM, NP, 5>(c, Ke, Kf, rhoJ, x, xidx, ld, base, bidx, bld, y, scale, ns);
         default: return cudaErrorInvalidValue;
     }

@@ -8,8 +8,9 @@
 // a shot and element costs 1,728 products instead of 4,050 and no vector is updated in memory: the
 // off-diagonal part of 64 shots on 12,544 triangles takes 139 us (282 us with the face and mass
 // kernels), of 32 shots on 4,096 triangles 33 us (67 us), of 8 on 3,844 11.5 us (30 us).  Plain sums took 113, 25
-// and 9.4 us, with up to a third more error.  Bound by latency at eight warps an SM (registers and 21 KB of
-// ring a warp); shared-memory reads and the joins of the compensated sums come next.
+// and 9.4 us, with up to a third more error.  Bound by latency at eight warps an SM (0.12 of the warps: 254 registers and
+// 21 KB of ring a warp; 64 shots on 12,544 triangles: issue 0.45 busy, DRAM 0.33, L1 0.35 of their peaks, the longest
+// stall a fixed-latency dependency); shared-memory reads and the joins of the compensated sums come next.
 //
 // Every warp runs a ring of four slot buffers (the shots' rows and K; buffer = slot), filled by
 // cp.async three slots ahead across element boundaries: three neighbours, then the element's own

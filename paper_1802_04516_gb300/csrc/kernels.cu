@@ -426,9 +426,10 @@ cudaError_t launch_to_fp32(stdg_ctx* c) {
 // product reads its second operand from the constant bank and shared memory only transposes.  A warp
 // takes 32 consecutive rows, copied by cp.async in order into rows of an odd number of pieces (no bank
 // conflicts), one group ahead; the results leave through the same buffer with consecutive stores.
-// Bound by HBM at size.  200,704 triangles, p = p_gamma = 3: MASSNEW us against 70 us for a block per 16
-// elements with one thread per (k, a) row reading M_ref and the values from shared memory; 82,944
-// tetrahedra, p = p_gamma = 2: MASSNEW3 against 35 us.  Same sums in the same order.
+// 200,704 triangles, p = p_gamma = 3: 21.6 us against 70 us for a block per 16 elements with one thread per
+// (k, a) row reading M_ref and the values from shared memory; 82,944 tetrahedra, p = p_gamma = 2: 12.6 against 35 us.
+// Bound by the L1 data pipe that the transposes go through (0.67 of L1's peak in 2D) at 0.24 of the warps; half of the
+// bytes stay in L2 (DRAM at 0.45).  Same sums in the same order.
 template <int NP, int NG>
 struct MassTables { float M[NP * NP], T[NG * NG]; };
 
@@ -811,7 +812,8 @@ cudaError_t launch_apply_caller(stdg_ctx* c, double dt, const double* x, double*
 // against 181 + 12 us, face and mass kernel, on 82,944 tetrahedra), and 2D at p = p_gamma = 3, where they
 // are little faster (264 against 253 + 22 us, cold, on 200,704 triangles) and move the mixed slab of the sliver mesh by more
 // than two runs differ (its inner residual is met by a different iterate; single velocities by 3e-7).
-// Elsewhere they win at every size (2D p = 2: 117 against 238 us on 200,704 triangles).
+// Elsewhere they win at every size (2D p = 2: 117 against 238 us on 200,704 triangles).  All for one shot: batches of
+// the two shapes run the register face kernel and were not measured on couplings.
 // In 3D with one time node D~ is read for few products and the couplings only win while they stay in
 // L2 (CG iteration at p = 2: 60 against 61 us on 4,374 tetrahedra = 79 MB, 120 against 92 us on 10,368; p = 1:
 // 42 against 56 us at 30 MB, 153 against 140 us at 138 MB).

@@ -1,7 +1,7 @@
 // Face kernels of the Schur velocity operator with compile-time sizes (dimension d,
 // N_phi, N_gamma) for the production shapes; other shapes use the generic kernel in
 // kernels.cu.  Shapes without a tiled kernel run from the assembled couplings (coupling.cu) and come
-// here only when those do not fit the device.  Same arithmetic as the generic kernel (Eq. velocity.sys with Q~ = -D^T
+// here only when those do not fit their share of the memory or are turned off.  Same arithmetic as the generic kernel (Eq. velocity.sys with Q~ = -D^T
 // and the orthonormalised dual basis):
 //   g = sum_side D~_side^T v_side,  t = E_j : g,  h = scale * S t,  y_side += D~_side h.
 // One warp per face.  Lanes hold one column (gather) and one row (scatter) of the face's

@@ -128,7 +128,7 @@ struct stdg_ctx {
     // copy has the faces' blocks in both orientations
     double *d_Kf = nullptr, *d_Ke = nullptr;
     float *d_Kf32 = nullptr, *d_Ke32 = nullptr;
-    double coupling_share = 1.0 / 16;   // of the free memory, the most that they may take
+    double coupling_share = 1.0 / 6;   // of the free memory, the most that they may take
     int2* d_adj = nullptr;      // [e][dim + 1]: neighbour (-1 on the boundary), 2 face + side of e
 
     // ---- device: state (shot-major)

@@ -181,10 +181,10 @@ def test_recorded_operator_outlives_the_couplings():
     del junk
 
 
-@pytest.mark.parametrize("room,share,held", [(6, None, False), (30, None, True), (6, 0.5, True), (30, 0.0, False)])
+@pytest.mark.parametrize("room,share,held", [(4, None, False), (12, None, True), (4, 0.5, True), (12, 0.0, False)])
 def test_couplings_take_no_more_than_their_share_of_the_free_memory(room, share, held):
     # a mesh whose couplings are 1/room of the memory that is free when they are laid out (the rest stays for others):
-    # by default they may take 1/16 of it
+    # by default they may take 1/6 of it
     torch = need_gpu()
     w = _workload(2, 3, 3, n=120)
     x = np.random.default_rng(8).normal(size=w.n_elem * 80)
