@@ -19,8 +19,8 @@ namespace stdg {
 // p_gamma = 2: 642 us with the face and mass kernels, 410 us here; 40,000 at p = 2: 398 and 163 us).  K_ii and the r
 // side's K_lr^T are read by columns (consecutive across the threads), the l side's K_lr by pieces of
 // its rows; the two ways of loading differ between the elements of a warp, the products do not.
-// FP32: bound by the latency of K from memory (3D p = 3, 7,986 tetrahedra: 604 MB at 0.59 of the DRAM peak, 0.22 of the
-// warps resident, 7.7 of 9.9 cycles an instruction waits on a long scoreboard; L1 data pipe 0.39).  A thread has two
+// FP32: bound by the latency of K from memory (3D p = 3, 7,986 tetrahedra: 605 MB at 0.54 of the DRAM peak, 0.22 of the
+// warps resident, 6.9 of 9.5 cycles an instruction waits on a long scoreboard; L1 data pipe 0.37).  A thread has two
 // consecutive rows, so that one 16-byte read of the staged values feeds them all, and the faces' blocks are
 // kept in both orientations, so that every load is a vector load of consecutive columns (reading rows of
 // one copy cost a wavefront per lane).
