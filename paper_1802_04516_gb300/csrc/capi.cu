@@ -135,7 +135,7 @@ static int fit_mma_image(stdg_ctx* c) {
     return STDG_OK;
 }
 
-static int alloc_state(stdg_ctx* c, int n_shots) {
+static int alloc_state_parts(stdg_ctx* c, int n_shots) {
     dev_free(c, c->d_vtr);
     dev_free(c, c->d_sigtr);
     dev_free(c, c->d_energy);
@@ -162,6 +162,21 @@ static int alloc_state(stdg_ctx* c, int n_shots) {
     solver_invalidate_graph(c);
     if ((rc = fit_mma_image(c)) != STDG_OK) return rc;
     return solver_setup(c);   // stacked Krylov workspace sized for n_shots
+}
+
+// State, records and Krylov workspace for n_shots.  Where one of them does not fit, all are given back: the
+// calls that need them then fail with STDG_ESTATE until a later stdg_set_shots succeeds.
+static int alloc_state(stdg_ctx* c, int n_shots) {
+    const int rc = alloc_state_parts(c, n_shots);
+    if (rc == STDG_OK) return rc;
+    solver_free(c);
+    for (void* p : {(void*)c->d_vtr, (void*)c->d_sigtr, (void*)c->d_energy, c->d_p2y, c->d_p2t, (void*)c->d_records}) dev_free(c, p);
+    c->d_vtr = c->d_sigtr = c->d_energy = c->d_records = nullptr;
+    c->d_p2y = c->d_p2t = nullptr;
+    c->rec_cap_steps = 0;
+    c->rec_steps = 0;
+    c->have_sources = 0;
+    return rc;
 }
 
 static int ensure_fp32(stdg_ctx* c) {
@@ -338,6 +353,7 @@ int take_device_error(stdg_ctx* c) {
 #define CHECK_CTX(c) do { if (!(c)) return STDG_EINVAL; } while (0)
 #define NEED_MESH(c) do { if (!(c)->have_mesh) STDG_FAIL(c, STDG_ESTATE, "call stdg_set_mesh first"); } while (0)
 #define NEED_ALL(c) do { NEED_MESH(c); if (!(c)->have_material) STDG_FAIL(c, STDG_ESTATE, "call stdg_set_material first"); } while (0)
+#define NEED_STATE(c) do { if (!(c)->d_vtr) STDG_FAIL(c, STDG_ESTATE, "no state (its allocation failed): call stdg_set_shots"); } while (0)
 
 extern "C" {
 
@@ -558,10 +574,10 @@ int stdg_set_mesh(stdg_ctx* c, int64_t n_vert, const double* xyz, int64_t n_elem
     c->d_Mdual = nullptr;
 #undef ALLOC
 #undef UP
-    c->have_mesh = true;
     if ((rc = alloc_state(c, 1)) != STDG_OK) return rc;
     if (c->opt.precision != STDG_FP64 && (rc = ensure_fp32(c)) != STDG_OK) return rc;
     STDG_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->have_mesh = true;
     return STDG_OK;
 }
 
@@ -587,7 +603,7 @@ int stdg_set_material(stdg_ctx* c, const double* lambda, const double* mu, const
 // dual cell (|T_{i,j}| = |T_i| / (d+1)), rho_i |J_i| per element; with a time scale alpha
 // the device holds alpha lambda, alpha mu, rho / alpha (physical copies kept for the energy).
 // Sets up the preconditioner.
-static int upload_material(stdg_ctx* c) {
+static int upload_material_parts(stdg_ctx* c) {
     const int64_t ne = c->n_elem, nf = c->n_face;
     const bool ts = !c->alpha_e.empty();
     int rc;
@@ -631,6 +647,28 @@ static int upload_material(stdg_ctx* c) {
     if ((rc = setup_coupling(c)) != STDG_OK) return rc;
     if (c->opt.preconditioner) return setup_pre1(c);
     return STDG_OK;
+}
+
+// Where a part of it fails, the context is left without a material and without the preconditioner's arrays.
+static int upload_material(stdg_ctx* c) {
+    const int rc = upload_material_parts(c);
+    if (rc == STDG_OK) return rc;
+    c->have_material = false;
+    solver_invalidate_graph(c);
+    cudaStreamSynchronize(c->stream);
+    for (void* p : {(void*)c->d_lamf_ph, (void*)c->d_muf_ph, (void*)c->d_rhoJ_ph, (void*)c->d_preV, (void*)c->d_preLam, (void*)c->d_preB,
+                    (void*)c->d_preV32, (void*)c->d_preB32, (void*)c->d_preB32t, (void*)c->d_pre2, (void*)c->d_pre2_32,
+                    (void*)c->d_pre2_mma, c->d_pre2_16, (void*)c->d_pre2_scl, (void*)c->d_p2status})
+        dev_free(c, p);
+    c->d_lamf_ph = c->d_muf_ph = c->d_rhoJ_ph = nullptr;
+    c->d_preV = c->d_preLam = c->d_preB = nullptr;
+    c->d_preV32 = c->d_preB32 = c->d_preB32t = nullptr;
+    c->d_pre2 = nullptr;
+    c->d_pre2_32 = c->d_pre2_mma = c->d_pre2_scl = nullptr;
+    c->d_pre2_16 = nullptr;
+    c->d_p2status = nullptr;
+    c->pre_dt = c->mma_dt = -1.0;
+    return rc;
 }
 
 // time scale of each point source: that of its element
@@ -679,6 +717,7 @@ int stdg_set_shots(stdg_ctx* c, int n_shots) {
 int stdg_set_state(stdg_ctx* c, int shot, const double* v_tr, const double* sig_tr) {
     CHECK_CTX(c);
     NEED_MESH(c);
+    NEED_STATE(c);
     if (shot < 0 || shot >= c->n_shots || !v_tr || !sig_tr) STDG_FAIL(c, STDG_EINVAL, "bad shot or null state");
     if (!all_finite(v_tr, c->ntr) || !all_finite(sig_tr, c->nsig)) STDG_FAIL(c, STDG_EINVAL, "non-finite state");
     STDG_CUDA(c, cudaMemcpyAsync(c->d_vtr + shot * c->ntr, v_tr, sizeof(double) * c->ntr, cudaMemcpyHostToDevice, c->stream));
@@ -692,6 +731,7 @@ int stdg_set_state(stdg_ctx* c, int shot, const double* v_tr, const double* sig_
 int stdg_get_state(stdg_ctx* c, int shot, double* v_tr, double* sig_tr) {
     CHECK_CTX(c);
     NEED_MESH(c);
+    NEED_STATE(c);
     if (shot < 0 || shot >= c->n_shots) STDG_FAIL(c, STDG_EINVAL, "bad shot");
     if (v_tr) STDG_CUDA(c, cudaMemcpyAsync(v_tr, c->d_vtr + shot * c->ntr, sizeof(double) * c->ntr, cudaMemcpyDeviceToHost, c->stream));
     if (sig_tr) {
@@ -705,6 +745,7 @@ int stdg_get_state(stdg_ctx* c, int shot, double* v_tr, double* sig_tr) {
 int stdg_set_plane_wave(stdg_ctx* c, int shot, int kind, const double* n, const double* pol, double amp, double t) {
     CHECK_CTX(c);
     NEED_ALL(c);
+    NEED_STATE(c);
     if (shot < 0 || shot >= c->n_shots || !n || (kind != 0 && kind != 1)) STDG_FAIL(c, STDG_EINVAL, "bad plane-wave arguments");
     if (!all_finite(n, c->dim) || (pol && !all_finite(pol, c->dim)) || !std::isfinite(amp) || !std::isfinite(t))
         STDG_FAIL(c, STDG_EINVAL, "non-finite plane-wave argument");
@@ -739,22 +780,24 @@ int stdg_set_point_sources(stdg_ctx* c, int n_shots, int per_shot, const double*
     if (!all_finite(xs, ns * d) || !all_finite(dir, ns * d) || !std::isfinite(f0) || !std::isfinite(t_delay) ||
         !std::isfinite(a1))
         STDG_FAIL(c, STDG_EINVAL, "non-finite source argument");
-    int rc = alloc_state(c, n_shots);
-    if (rc != STDG_OK) return rc;
     std::vector<double> host((size_t)ns * (d + NP));
-    c->src_elem.assign(ns, 0);
+    std::vector<int64_t> elem(ns);
     for (int64_t s = 0; s < ns; ++s) {
         double y[3];
         int64_t e = locate_point(c->hm, xs + s * d, y);
         if (e < 0) STDG_FAIL(c, STDG_EINVAL, "source outside the mesh");
-        c->src_elem[s] = e;
+        elem[s] = e;
         for (int a = 0; a < d; ++a) host[s * (d + NP) + a] = dir[s * d + a];
         eval_phi_host(c, e, y, &host[s * (d + NP) + d]);
     }
+    c->have_sources = 0;   // until the arrays of the new ones are there
+    int rc = alloc_state(c, n_shots);
+    if (rc != STDG_OK) return rc;
     dev_free(c, c->d_src);
     c->d_src = nullptr;
     if ((rc = dev_alloc(c, (void**)&c->d_src, sizeof(double) * host.size())) != STDG_OK) return rc;
     STDG_CUDA(c, cudaMemcpy(c->d_src, host.data(), sizeof(double) * host.size(), cudaMemcpyHostToDevice));
+    c->src_elem = elem;
     c->src_per_shot = per_shot;
     c->src_xs.assign(xs, xs + ns * d);
     c->src_dir.assign(dir, dir + ns * d);
@@ -791,7 +834,7 @@ int stdg_set_receivers(stdg_ctx* c, int n_rec, const double* xr) {
     dev_free(c, c->d_records);
     c->d_rec_elem = nullptr;
     c->d_rec_phi = c->d_records = nullptr;
-    c->n_rec = n_rec;
+    c->n_rec = 0;   // until their arrays are there
     c->rec_steps = 0;
     c->rec_cap_steps = 0;
     solver_invalidate_graph(c);
@@ -799,6 +842,7 @@ int stdg_set_receivers(stdg_ctx* c, int n_rec, const double* xr) {
     int rc;
     if ((rc = dev_alloc(c, (void**)&c->d_rec_elem, sizeof(int32_t) * n_rec)) != STDG_OK) return rc;
     if ((rc = dev_alloc(c, (void**)&c->d_rec_phi, sizeof(double) * n_rec * NP)) != STDG_OK) return rc;
+    c->n_rec = n_rec;
     STDG_CUDA(c, cudaMemcpy(c->d_rec_elem, el.data(), sizeof(int32_t) * n_rec, cudaMemcpyHostToDevice));
     STDG_CUDA(c, cudaMemcpy(c->d_rec_phi, phi.data(), sizeof(double) * n_rec * NP, cudaMemcpyHostToDevice));
     return STDG_OK;
@@ -827,6 +871,7 @@ static int ensure_records(stdg_ctx* c, int n_steps) {
 int stdg_step(stdg_ctx* c, double dt, int n_steps, stdg_stats* out) {
     CHECK_CTX(c);
     NEED_ALL(c);
+    NEED_STATE(c);
     if (!(dt > 0) || !std::isfinite(dt) || n_steps < 0) STDG_FAIL(c, STDG_EINVAL, "dt must be > 0 and n_steps >= 0");
     if (out) std::memset(out, 0, sizeof(*out));
     if (n_steps == 0) return STDG_OK;
@@ -900,6 +945,7 @@ int stdg_set_time(stdg_ctx* c, double t) {
 int stdg_energy(stdg_ctx* c, double* out) {
     CHECK_CTX(c);
     NEED_ALL(c);
+    NEED_STATE(c);
     if (!out) return STDG_EINVAL;
     for (int s = 0; s < c->n_shots; ++s) {
         STDG_CUDA(c, launch_energy(c, s, c->d_energy + s));

@@ -212,3 +212,74 @@ def test_non_finite_residual_of_a_finite_right_hand_side_ends_the_restarts(preci
             alone.set_state(*states[k])
             alone.step(dt, 1)
             assert rel_l2(s.get_state(k)[0], alone.get_state()[0]) < 1e-7
+
+
+def test_state_that_does_not_fit_leaves_the_calls_refused():
+    # a shot count whose state cannot be allocated (hundreds of GB): the calls that need it are refused, nothing runs on
+    # missing arrays, and the context works again with a count that fits
+    need_gpu()
+    from paper_1802_04516_gb300.binding import STDG_ENOMEM, STDG_ESTATE, StdgError
+    w = _small()
+    fresh = gpu_solver(w, precision="mixed", rel_tol=1e-10, max_iters=20000, preconditioner=2)
+    fresh.step(w.dt, 2)
+    s = gpu_solver(w, precision="mixed", rel_tol=1e-10, max_iters=20000, preconditioner=2)
+    s.step(w.dt, 1)
+    v, sig = s.get_state()
+    with pytest.raises(StdgError) as ei:
+        s.set_shots(1 << 27)
+    assert ei.value.code == STDG_ENOMEM
+    for call in (lambda: s.step(w.dt, 1), lambda: s.get_state(), lambda: s.set_state(v, sig), lambda: s.energy(),
+                 lambda: s.set_plane_wave(0, [1.0, 0.0], amp=0.1)):
+        with pytest.raises(StdgError) as ei:
+            call()
+        assert ei.value.code == STDG_ESTATE
+    s.set_sources(w.shots_xs, w.shots_dir, w.f0, w.t_delay, w.a1)
+    s.time = 0.0
+    assert s.step(w.dt, 2)["status"] == 0
+    assert rel_l2(s.get_state()[0], fresh.get_state()[0]) < 1e-8
+
+
+@pytest.mark.parametrize("pre", [1, 2])
+def test_material_that_does_not_fit_leaves_the_calls_refused(pre):
+    # the memory is taken by another library when the material is set: no room for the preconditioner's blocks
+    torch = need_gpu()
+    from paper_1802_04516_gb300.binding import STDG_ENOMEM, STDG_ESTATE, Solver, StdgError
+    xyz, ev, per = synth.tri_grid(121, 120, 1.0, 1.0, periodic=False, jitter=0.2, seed=3)
+    medium = synth.homogeneous(ev.shape[0], 2.0, 1.0, 1.0)
+    s = Solver(2, 3, 3, rel_tol=1e-8, max_iters=5000, preconditioner=pre)
+    s.set_mesh(xyz, ev, per)
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    fill = torch.empty(free - (32 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(StdgError) as ei:
+            s.set_material(*medium)
+        assert ei.value.code == STDG_ENOMEM
+        for call in (lambda: s.step(1e-3, 1), lambda: s.apply_operator(1e-3, np.zeros(s.nvel)),
+                     lambda: s.apply_preconditioner(1e-3, np.zeros(s.nvel))):
+            with pytest.raises(StdgError) as ei:
+                call()
+            assert ei.value.code == STDG_ESTATE
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    s.set_material(*medium)
+    v, sig = s.get_state()
+    s.set_state(v + 1.0, sig)
+    assert s.step(1e-3, 1)["status"] == 0
+
+
+def test_rejected_sources_leave_the_state_and_the_sources():
+    need_gpu()
+    from paper_1802_04516_gb300.binding import STDG_EINVAL, StdgError
+    w = _small()
+    a, b = (gpu_solver(w, rel_tol=1e-12, max_iters=20000) for _ in range(2))
+    for s in (a, b):
+        s.step(w.dt, 1)
+    outside = np.concatenate([np.array(w.shots_xs, dtype=float), [[-5.0, -5.0]] * 3])
+    with pytest.raises(StdgError) as ei:
+        a.set_sources(outside, np.tile([0.0, 1.0], (4, 1)), w.f0, w.t_delay, w.a1)
+    assert ei.value.code == STDG_EINVAL and a.query(6) == 1
+    for s in (a, b):
+        s.step(w.dt, 1)
+    assert rel_l2(a.get_state()[0], b.get_state()[0]) < 1e-10
